@@ -168,10 +168,6 @@ struct feti_ctx {
   std::vector<int32_t> env0;
   std::vector<int64_t> env_off;
   int32_t* d_env0 = nullptr;
-  // the same for the FP32 elimination's kChol32Block-column steps
-  std::vector<int32_t> env0_32;
-  std::vector<int64_t> env32_off;
-  int32_t* d_env0_32 = nullptr;
   // local factorizations in groups: subdomains [grp[g], grp[g + 1]) are
   // eliminated together in the one workspace d_A / d_A32 of ws_elems
   // elements (ws_full: every subdomain at once); d_lay_ws holds the layouts
@@ -180,6 +176,8 @@ struct feti_ctx {
   // compact interior factor d_Lc / d_Lc32 (lc_elems) serves every K^+.
   std::vector<int32_t> grp;
   SubLayout* d_lay_ws = nullptr;
+  int64_t chol_scratch = 0;  // bytes of the elimination scratch (digit slices of a step's panel), largest group
+  uint8_t* d_cholz = nullptr;
   int64_t ws_elems = 0, ws_full = 0, lc_elems = 0;
   bool keep_factor = false;
   double* d_Lc = nullptr;
@@ -677,7 +675,6 @@ feti_status build_decomposition(feti_ctx* ctx) {
   // per subdomain: free DOFs, kernels, fixing DOFs, dense order
   ctx->lay.assign(P, SubLayout{});
   std::vector<std::vector<int32_t>> env0(P);  // per interior-elimination step: (eI, nbact)
-  std::vector<std::vector<int32_t>> env0w(P);  // the same for kChol32Block-column steps
   ctx->fix_ptr.assign(P + 1, 0);
   ctx->fix_ldof.clear();
   std::vector<std::vector<int32_t>> dense_ldof(P);  // dense index -> local DOF
@@ -844,14 +841,10 @@ feti_status build_decomposition(feti_ctx* ctx) {
       for (int v = 1; v <= nI; ++v) last[v] = std::max(last[v], last[v - 1]);
       std::vector<int32_t> bfirst(nbp);
       for (int i = 0; i < nbp; ++i) bfirst[i] = dof_first[bsort[i]];
-      for (int w = 0; w < 2; ++w) {
-        auto& ev = w == 0 ? env0[s] : env0w[s];
-        const int B = w == 0 ? 32 : feti::kChol32Block;
-        for (int kb = 0; kb < nI; kb += B) {
-          const int r0 = kb + std::min(B, nI - kb);
-          ev.push_back(std::max(r0, last[r0] + 1));
-          ev.push_back((int32_t)(std::lower_bound(bfirst.begin(), bfirst.end(), r0) - bfirst.begin()));
-        }
+      for (int kb = 0; kb < nI; kb += feti::kCholPanel) {
+        const int r0 = kb + std::min(feti::kCholPanel, nI - kb);
+        env0[s].push_back(std::max(r0, last[r0] + 1));
+        env0[s].push_back((int32_t)(std::lower_bound(bfirst.begin(), bfirst.end(), r0) - bfirst.begin()));
       }
     }
     for (int d : fix) dl.push_back(d);
@@ -933,8 +926,16 @@ feti_status build_decomposition(feti_ctx* ctx) {
   }
   const int n_grp = (int)ctx->grp.size() - 1;
   std::vector<SubLayout> lay_ws(ctx->lay);
-  for (int g = 0; g < n_grp; ++g)
-    for (int s = ctx->grp[g]; s < ctx->grp[g + 1]; ++s) lay_ws[s].aoff -= ctx->lay[ctx->grp[g]].aoff;
+  ctx->chol_scratch = 0;
+  for (int g = 0; g < n_grp; ++g) {
+    int64_t z = 0;  // elimination scratch of the group
+    for (int s = ctx->grp[g]; s < ctx->grp[g + 1]; ++s) {
+      lay_ws[s].aoff -= ctx->lay[ctx->grp[g]].aoff;
+      lay_ws[s].zoff = z;
+      z += feti::chol_scratch_bytes(lay_ws[s].n, ctx->opt.precision == FETI_MIXED_F32FACTOR ? 4 : 8);
+    }
+    ctx->chol_scratch = std::max(ctx->chol_scratch, z);
+  }
   FETI_TRY(upload(ctx, &ctx->d_lay_ws, lay_ws));
   // envelope tables of the interior elimination, [step][subdomain of the group][2] per group
   auto env_tables = [&](const std::vector<std::vector<int32_t>>& ev, std::vector<int32_t>& tab,
@@ -956,10 +957,6 @@ feti_status build_decomposition(feti_ctx* ctx) {
   };
   env_tables(env0, ctx->env0, ctx->env_off);
   FETI_TRY(upload(ctx, &ctx->d_env0, ctx->env0));
-  if (ctx->opt.precision == FETI_MIXED_F32FACTOR) {
-    env_tables(env0w, ctx->env0_32, ctx->env32_off);
-    FETI_TRY(upload(ctx, &ctx->d_env0_32, ctx->env0_32));
-  }
   for (const auto& L : ctx->lay) ctx->max_nr = std::max(ctx->max_nr, L.nI + L.nbp);
   ctx->nloc_total = voff;
   ctx->cd = coff;
@@ -1481,6 +1478,7 @@ feti_status check_status(feti_ctx* ctx, const char* where) {
     FETI_CK(cudaStreamSynchronize(ctx->stream));
   }
   if (s == feti::DEV_LOCAL_SINGULAR) return fail(ctx, FETI_ERR_LOCAL_SINGULAR, std::string(where) + ": non-positive pivot");
+  if (s == feti::DEV_TIMEOUT) return fail(ctx, FETI_ERR_TIMEOUT, std::string(where) + ": a bounded wait ran out");
   if (s == feti::DEV_INVERTED) return fail(ctx, FETI_ERR_ELEMENT_INVERTED, std::string(where) + ": inverted element");
   if (s != 0) return fail(ctx, FETI_ERR_CUDA, std::string(where) + ": device status " + std::to_string(s));
   return FETI_OK;
@@ -1653,15 +1651,14 @@ feti_status tune_refinement(feti_ctx* ctx) {
 // interior factor.  T is the factorization's precision.  Returns the first
 // error of the enqueueing calls.
 template <typename T>
-cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, const std::vector<int32_t>& envt, const std::vector<int64_t>& eoff,
-                     const int32_t* d_env, int B, double* S64, float* S32,
-                     float* S32s, double* F64, float* F32, float* F32s, T* Lc) {
+cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, double* S64, float* S32, float* S32s, double* F64, float* F32,
+                            float* F32s, T* Lc) {
   cudaStream_t st = ctx->stream;
   const int s0 = ctx->grp[g], pg = ctx->grp[g + 1] - s0;
   const SubLayout* lw = ctx->d_lay_ws + s0;
   int64_t elems = 0;
   for (int s = s0; s < s0 + pg; ++s) elems += (int64_t)ctx->lay[s].ld * ctx->lay[s].ld;
-  const cudaError_t e = cudaMemsetAsync(A, 0, (size_t)elems * sizeof(T), st);
+  cudaError_t e = cudaMemsetAsync(A, 0, (size_t)elems * sizeof(T), st);
   if (e != cudaSuccess) return e;
   feti::launch_assemble(pg, lw, ctx->d_sub_elem_ptr + s0, ctx->d_sub_elems, ctx->d_elem_dense, ctx->d_Ke, ctx->nde,
                         A, st);
@@ -1673,9 +1670,9 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, const std::vector<int32_
     const int64_t i0 = ctx->lump_grp[g], i1 = ctx->lump_grp[g + 1];
     feti::launch_lump_fill((long)(i1 - i0), ctx->d_lump_src + i0, A, ctx->d_lump_val + i0, st);
   }
-  // per step, the largest trailing chunk count over the group's subdomains
-  // (steps of B columns)
-  std::vector<int> chunks[2];
+  // per step, the largest number of active rows over the group's subdomains
+  constexpr int B = feti::kCholPanel;
+  std::vector<int> rows[2];
   for (int phase = 0; phase < 2; ++phase)
     for (int s = s0; s < s0 + pg; ++s) {
       const SubLayout& L = ctx->lay[s];
@@ -1687,21 +1684,23 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, const std::vector<int32_
         // rows plus the augmentation rows of the columns eliminated so far
         int m;
         if (phase == 0) {
-          const int32_t* ev = &envt[eoff[g] + 2 * ((size_t)t * pg + (s - s0))];
+          const int32_t* ev = &ctx->env0[ctx->env_off[g] + 2 * ((size_t)t * pg + (s - s0))];
           m = (ev[0] - r0) + ev[1] + L.k;
         } else {
           m = std::min(L.ld, L.n + r0 - L.nI) - r0;
         }
-        const int ch = (m + 63) / 64;
-        if ((int)chunks[phase].size() <= t) chunks[phase].push_back(0);
-        chunks[phase][t] = std::max(chunks[phase][t], ch);
+        if ((int)rows[phase].size() <= t) rows[phase].push_back(0);
+        rows[phase][t] = std::max(rows[phase][t], m);
       }
     }
-  feti::launch_chol_batched(pg, lw, 0, chunks[0].data(), (int)chunks[0].size(), d_env + eoff[g], A, ctx->d_status,
-                            st);
+  e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g], A,
+                                ctx->d_cholz, ctx->d_status, st);
+  if (e != cudaSuccess) return e;
   if (ctx->opt.precond == FETI_PREC_DIRICHLET)
     feti::launch_extract_tiles(pg, ctx->max_nb, lw, 0, A, S64, S32, S32s, st);
-  feti::launch_chol_batched(pg, lw, 1, chunks[1].data(), (int)chunks[1].size(), nullptr, A, ctx->d_status, st);
+  e = feti::launch_chol_batched(pg, lw, 1, rows[1].data(), (int)rows[1].size(), nullptr, A, ctx->d_cholz,
+                                ctx->d_status, st);
+  if (e != cudaSuccess) return e;
   feti::launch_extract_tiles(pg, ctx->max_nb, lw, 1, A, F64, F32, F32s, st);
   if (Lc) feti::launch_compact_factor(pg, ctx->max_nr, lw, A, Lc, st);
   return cudaGetLastError();
@@ -1712,8 +1711,7 @@ feti_status factorize_all(feti_ctx* ctx) {
   if (f32_factor(ctx)) {
     // FP32 elimination; S_i and F_i go straight into the FP32 operator layouts
     for (int g = 0; g < n_grp; ++g)
-      FETI_CK(factorize_group<float>(ctx, g, ctx->d_A32, ctx->env0_32, ctx->env32_off, ctx->d_env0_32,
-                             feti::kChol32Block, nullptr, ctx->d_S32, ctx->d_S32s, nullptr, ctx->d_F32, ctx->d_F32s,
+      FETI_CK(factorize_group<float>(ctx, g, ctx->d_A32, nullptr, ctx->d_S32, ctx->d_S32s, nullptr, ctx->d_F32, ctx->d_F32s,
                              ctx->d_Lc32));
     FETI_TRY(check_status(ctx, "local factorization (FP32)"));
     return FETI_OK;
@@ -1721,7 +1719,7 @@ feti_status factorize_all(feti_ctx* ctx) {
   // FP64 operators, and in the FP32-local form their FP32 copies, in one pass each
   const bool mix = ctx->opt.precision == FETI_MIXED;
   for (int g = 0; g < n_grp; ++g)
-    FETI_CK(factorize_group<double>(ctx, g, ctx->d_A, ctx->env0, ctx->env_off, ctx->d_env0, 32, ctx->d_S,
+    FETI_CK(factorize_group<double>(ctx, g, ctx->d_A, ctx->d_S,
                             mix ? ctx->d_S32 : nullptr, mix ? ctx->d_S32s : nullptr, ctx->d_F,
                             mix ? ctx->d_F32 : nullptr, mix ? ctx->d_F32s : nullptr,
                             ctx->keep_factor ? nullptr : ctx->d_Lc));
@@ -2195,6 +2193,7 @@ feti_status build_pcg_graph(feti_ctx* ctx, int chunk, bool mixed) {
 // Dense local matrices (factorized in place), S_i, F_i and their FP32 copies.
 feti_status alloc_operators(feti_ctx* ctx) {
   if (ctx->d_A || ctx->d_A32) return FETI_OK;
+  FETI_TRY(dev_alloc(ctx, &ctx->d_cholz, (size_t)ctx->chol_scratch));
   if (f32_factor(ctx)) {
     FETI_TRY(dev_alloc(ctx, &ctx->d_A32, (size_t)ctx->op_elems[0]));
     FETI_TRY(dev_alloc(ctx, &ctx->d_kr, (size_t)ctx->nloc_total));

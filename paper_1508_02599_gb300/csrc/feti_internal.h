@@ -16,6 +16,7 @@ enum DevStatus : int {
   DEV_LOCAL_SINGULAR = 1,   // non-positive pivot in a local Cholesky factorization
   DEV_INVERTED = 2,         // element with non-positive volume or det F
   DEV_BREAKDOWN = 3,        // (p, F p) <= 0 or not finite
+  DEV_TIMEOUT = 4,          // a bounded wait of the factorization kernels ran out
 };
 
 // Per-subdomain dense layout.  Dense local order: [interior | boundary minus
@@ -46,6 +47,7 @@ struct SubLayout {
   int64_t psym;   // offset (floats) of the transposed-product partials: PH I floats per panel I
   int64_t loff;   // offset of the compact interior factor: rows [0, nI + nbp) x columns [0, nI)
                   // of the Cholesky factor (L_II lower, L_bI), row stride kp_ld
+  int64_t zoff;   // offset (bytes) of the elimination scratch, relative to the group's first
 };
 // Row stride of the compact interior factor (a multiple of 4 elements).
 __host__ __device__ inline int kp_ld(const SubLayout& L) { return (L.nI + 3) & ~3; }
@@ -273,27 +275,23 @@ void launch_spmv_lump(int n_rows, const int32_t* ptr, const int32_t* col, const 
 }  // namespace feti
 
 namespace feti {
-// Batched multi-CTA partial Cholesky of every subdomain's dense matrix, one
-// launch triple (diagonal block, panel solve, tiled trailing update) per
-// 32-column step; phase 0: interior columns, phase 1: boundary minus fixing
-// columns.  Each step updates only the rows its block column can reach:
-// phase 0 the envelope given by env0 ([step][subdomain] pairs (eI, nbact):
-// interior rows up to eI, the first nbact boundary rows, the fixing rows),
-// phase 1 the remaining rows plus the augmentation rows of the columns
-// eliminated so far (env0 unused).  step_chunks[t] (host array, n_steps
-// entries): the largest number of 64-row chunks of those rows over the
-// subdomains at step t (idle CTAs exit at once).
-void launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_chunks, int n_steps,
-                         const int32_t* env0, double* A, int* status, cudaStream_t st);
-// The same steps on the FP32 workspace (FP32 factorization), in blocks of
-// kChol32Block columns (the step and envelope tables use that width).  64
-// columns halve the passes over the trailing matrix (112 against 140 ms of
-// elimination on the 1024-subdomain tube) but the FP32 factor then needs one
-// more refinement correction and three more inner PCG iterations, which
-// costs more than it saves: 32.
-constexpr int kChol32Block = 32;
-void launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_chunks, int n_steps,
-                         const int32_t* env0, float* A, int* status, cudaStream_t st);
+// Batched multi-CTA partial Cholesky of every subdomain's dense matrix
+// (feti_chol_tc.cu), three launches (diagonal block, panel solve, tiled
+// trailing update) per kCholPanel-column step; phase 0: interior columns,
+// phase 1: boundary minus fixing columns.  Each step updates only the rows
+// its block column can reach: phase 0 the envelope given by env0
+// ([step][subdomain] pairs (eI, nbact): interior rows up to eI, the first
+// nbact boundary rows, the fixing rows), phase 1 the remaining rows plus the
+// augmentation rows of the columns eliminated so far (env0 unused).
+// step_rows[t] (host array, n_steps entries): the largest number of those rows
+// over the subdomains at step t.  Z: scratch, chol_scratch_bytes per subdomain
+// at SubLayout::zoff.
+constexpr int kCholPanel = 64;
+int64_t chol_scratch_bytes(int n, int elem_bytes);
+cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
+                                const int32_t* env0, double* A, uint8_t* Z, int* status, cudaStream_t st);
+cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
+                                const int32_t* env0, float* A, uint8_t* Z, int* status, cudaStream_t st);
 }  // namespace feti
 
 namespace feti {

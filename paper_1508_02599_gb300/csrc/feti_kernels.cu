@@ -2081,254 +2081,6 @@ void launch_spmv_lump(int n_rows, const int32_t* ptr, const int32_t* col, const 
 }
 
 namespace {
-// Batched multi-CTA partial Cholesky: one launch per block-column step for
-// all subdomains together (blockIdx.y = subdomain).  Phase 0 eliminates the
-// interior columns [0, nI) with trailing rows/cols [.., n); phase 1 the
-// boundary columns [nI, nI + nbp) with trailing rows/cols [.., ld).
-struct PhaseRange {
-  int c0, c1;
-};
-__device__ __forceinline__ PhaseRange phase_range(const SubLayout& L, int phase) {
-  return phase == 0 ? PhaseRange{0, L.nI} : PhaseRange{L.nI, L.nI + L.nbp};
-}
-// Rows that block column [kb, kb + nk) can change, as an increasing map of
-// 0 .. m - 1 onto matrix rows; the rows left out would receive exact zeros.
-// Phase 0 (envelope of the interior columns: a row is zero left of the first
-// interior column it couples to, and Cholesky fill stays inside that
-// envelope): interior rows r0 .. eI - 1, the first nbact boundary rows (the
-// boundary DOFs are ordered by envelope start) and the fixing rows, with
-// (eI, nbact) per step and subdomain from the host.  Phase 1: rows r0 .. n - 1
-// and the augmentation rows of the columns eliminated so far (augmentation
-// row n + a starts as the unit row of column nI + a and stays zero left of
-// that column until it is eliminated).
-struct ActiveRows {
-  int r0, lenA, lenB, bbase, cbase, m;
-  __device__ __forceinline__ int row(int q) const {
-    return q < lenA ? r0 + q : (q < lenA + lenB ? bbase + (q - lenA) : cbase + (q - lenA - lenB));
-  }
-};
-__device__ __forceinline__ ActiveRows active_rows(const SubLayout& L, int phase, int step, int kb, int nk,
-                                                  const int32_t* __restrict__ env0) {
-  ActiveRows a;
-  a.r0 = kb + nk;
-  if (phase == 0) {
-    const int32_t* ev = env0 + 2 * ((size_t)step * gridDim.y + blockIdx.y);
-    const int eI = min(max(ev[0], a.r0), L.nI);
-    const int nbact = min(max(ev[1], 0), L.nbp);
-    a.lenA = eI - a.r0;
-    a.lenB = nbact;
-    a.bbase = L.nI;
-    a.cbase = L.nI + L.nbp;
-    a.m = a.lenA + a.lenB + L.k;
-  } else {
-    a.lenA = min(L.ld, L.n + a.r0 - L.nI) - a.r0;
-    a.lenB = 0;
-    a.bbase = a.cbase = a.r0;
-    a.m = a.lenA;
-  }
-  return a;
-}
-
-template <typename T, int B>
-__global__ void k_bat_diag(const SubLayout* __restrict__ lay, int phase, int step, T* __restrict__ Abase,
-                           int* status) {
-  const SubLayout L = lay[blockIdx.y];
-  const PhaseRange pr = phase_range(L, phase);
-  const int kb = pr.c0 + step * B;
-  if (kb >= pr.c1) return;
-  const int nk = min(B, pr.c1 - kb);
-  T* A = Abase + L.aoff;
-  const size_t ld = L.ld;
-  __shared__ T D[B][B + 1];
-  __shared__ int bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) bad = 0;
-  for (int idx = tid; idx < B * B; idx += blockDim.x) {
-    const int i = idx / B, j = idx % B;
-    D[i][j] = (i < nk && j <= i) ? A[(kb + i) * ld + kb + j] : (T)0;
-  }
-  __syncthreads();
-  if (B == 32) {
-    if (tid < 32) {
-      const int i = tid;
-      for (int j = 0; j < nk; ++j) {
-        if (i == j) {
-          const T d = D[j][j];
-          if (!(d > 0.0) || !isfinite(d)) bad = 1;
-          D[j][j] = sqrt(d);
-        }
-        __syncwarp();
-        if (bad) break;
-        if (i > j && i < nk) D[i][j] /= D[j][j];
-        __syncwarp();
-        if (i > j && i < nk)
-          for (int l = j + 1; l <= i; ++l) D[i][l] -= D[i][j] * D[l][j];
-        __syncwarp();
-      }
-    }
-  } else {
-    // wider blocks: row i by thread i, every thread through the block barriers
-    const int i = tid;
-    for (int j = 0; j < nk; ++j) {
-      if (i == j) {
-        const T d = D[j][j];
-        if (!(d > 0.0) || !isfinite(d)) bad = 1;
-        D[j][j] = sqrt(d);
-      }
-      __syncthreads();
-      if (bad) break;
-      if (i > j && i < nk) D[i][j] /= D[j][j];
-      __syncthreads();
-      if (i > j && i < nk)
-        for (int l = j + 1; l <= i; ++l) D[i][l] -= D[i][j] * D[l][j];
-      __syncthreads();
-    }
-  }
-  __syncthreads();
-  if (bad) {
-    if (tid == 0) set_status(status, DEV_LOCAL_SINGULAR);
-    return;
-  }
-  for (int idx = tid; idx < nk * nk; idx += blockDim.x) {
-    const int i = idx / nk, j = idx % nk;
-    if (j <= i) A[(kb + i) * ld + kb + j] = D[i][j];
-  }
-}
-
-template <typename T, int B>
-__global__ void k_bat_trsm(const SubLayout* __restrict__ lay, int phase, int step,
-                           const int32_t* __restrict__ env0, T* __restrict__ Abase, const int* status) {
-  if (*status) return;
-  const SubLayout L = lay[blockIdx.y];
-  const PhaseRange pr = phase_range(L, phase);
-  const int kb = pr.c0 + step * B;
-  if (kb >= pr.c1) return;
-  const int nk = min(B, pr.c1 - kb);
-  const ActiveRows ar = active_rows(L, phase, step, kb, nk, env0);
-  const int q0 = blockIdx.x * TT;
-  if (q0 >= ar.m) return;
-  const int nr = min(TT, ar.m - q0);
-  T* A = Abase + L.aoff;
-  const size_t ld = L.ld;
-  __shared__ T D[B][B + 1];
-  __shared__ T Pa[TT][B + 1];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < B * B; idx += blockDim.x) {
-    const int i = idx / B, j = idx % B;
-    D[i][j] = (i < nk && j <= i) ? A[(kb + i) * ld + kb + j] : (T)0;
-  }
-  for (int idx = tid; idx < TT * B; idx += blockDim.x) {
-    const int r = idx / B, l = idx % B;
-    Pa[r][l] = (r < nr && l < nk) ? A[(size_t)ar.row(q0 + r) * ld + kb + l] : (T)0;
-  }
-  __syncthreads();
-  if (tid < nr) {
-    T xr[B];
-#pragma unroll
-    for (int j = 0; j < B; ++j) xr[j] = Pa[tid][j];
-#pragma unroll
-    for (int j = 0; j < B; ++j) {
-      if (j < nk) {
-        T v = xr[j];
-#pragma unroll
-        for (int l = 0; l < B; ++l)
-          if (l < j) v -= xr[l] * D[j][l];
-        xr[j] = v / D[j][j];
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < B; ++j) Pa[tid][j] = xr[j];
-  }
-  __syncthreads();
-  for (int idx = tid; idx < TT * B; idx += blockDim.x) {
-    const int r = idx / B, l = idx % B;
-    if (r < nr && l < nk) A[(size_t)ar.row(q0 + r) * ld + kb + l] = Pa[r][l];
-  }
-}
-
-template <typename T, int B>
-__global__ void __launch_bounds__(kThreads) k_bat_update(const SubLayout* __restrict__ lay, int phase, int step,
-                                                         const int32_t* __restrict__ env0,
-                                                         T* __restrict__ Abase, const int* status) {
-  if (*status) return;
-  const SubLayout L = lay[blockIdx.y];
-  const PhaseRange pr = phase_range(L, phase);
-  const int kb = pr.c0 + step * B;
-  if (kb >= pr.c1) return;
-  const int nk = min(B, pr.c1 - kb);
-  const ActiveRows ar = active_rows(L, phase, step, kb, nk, env0);
-  const int m = ar.m;
-  const int chunks = (m + TT - 1) / TT;
-  const long b = blockIdx.x;
-  if (b >= (long)chunks * (chunks + 1) / 2) return;
-  int ti = (int)((sqrt(8.0 * (double)b + 1.0) - 1.0) * 0.5);
-  while ((long)(ti + 1) * (ti + 2) / 2 <= b) ++ti;
-  while ((long)ti * (ti + 1) / 2 > b) --ti;
-  const int tj = (int)(b - (long)ti * (ti + 1) / 2);
-  const int ib = ti * TT, jb = tj * TT;  // positions in the active-row list
-  T* A = Abase + L.aoff;
-  const size_t ld = L.ld;
-  __shared__ T Pa[TT][B + 1];
-  __shared__ T Pb[TT][B + 1];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < TT * B; idx += blockDim.x) {
-    const int r = idx / B, l = idx % B;
-    Pa[r][l] = (ib + r < m && l < nk) ? A[(size_t)ar.row(ib + r) * ld + kb + l] : (T)0;
-    Pb[r][l] = (jb + r < m && l < nk) ? A[(size_t)ar.row(jb + r) * ld + kb + l] : (T)0;
-  }
-  __syncthreads();
-  const int tr = (tid / 16) * 4, tc = (tid % 16) * 4;
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = (T)0;
-  for (int l = 0; l < nk; ++l) {
-    T av[4], bv[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      av[a] = Pa[tr + a][l];
-      bv[a] = Pb[tc + a][l];
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][c] += av[a] * bv[c];
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int qi = ib + tr + a, qj = jb + tc + c;  // increasing map: qj <= qi <=> j <= i
-      if (qi < m && qj < m && qj <= qi) A[(size_t)ar.row(qi) * ld + ar.row(qj)] -= acc[a][c];
-    }
-}
-}  // namespace
-
-template <typename T, int B>
-void chol_batched(int P, const SubLayout* lay, int phase, const int* step_chunks, int n_steps,
-                  const int32_t* env0, T* A, int* status, cudaStream_t st) {
-  for (int t = 0; t < n_steps; ++t) {
-    const int chunks = step_chunks[t];
-    k_bat_diag<T, B><<<dim3(1, P), kThreads, 0, st>>>(lay, phase, t, A, status);
-    if (chunks <= 0) continue;
-    k_bat_trsm<T, B><<<dim3(chunks, P), kThreads, 0, st>>>(lay, phase, t, env0, A, status);
-    const long tiles = (long)chunks * (chunks + 1) / 2;
-    k_bat_update<T, B><<<dim3((unsigned)tiles, P), kThreads, 0, st>>>(lay, phase, t, env0, A, status);
-  }
-}
-
-void launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_chunks, int n_steps,
-                         const int32_t* env0, double* A, int* status, cudaStream_t st) {
-  chol_batched<double, 32>(P, lay, phase, step_chunks, n_steps, env0, A, status, st);
-}
-
-void launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_chunks, int n_steps,
-                         const int32_t* env0, float* A, int* status, cudaStream_t st) {
-  chol_batched<float, kChol32Block>(P, lay, phase, step_chunks, n_steps, env0, A, status, st);
-}
-
-namespace {
 __global__ void k_ke_unpack(long n, int nde, const double* __restrict__ Kp, double* __restrict__ K) {
   const int kes = nde * nde;
   for (long x = blockIdx.x * (long)blockDim.x + threadIdx.x; x < n; x += (long)gridDim.x * blockDim.x) {

@@ -7,6 +7,7 @@
 // Scalars (rho, alpha, beta, norms) are per right-hand side; a converged
 // right-hand side is frozen (alpha = beta = 0 for it) while the others run on.
 #include "feti_internal.h"
+#include "feti_tc.cuh"
 
 #include <cuda.h>
 
@@ -447,32 +448,6 @@ __global__ void k_col_set(int n, int nrhs, int k, double scale, const double* __
 // global loads map onto conflict-free shared-memory stores.  One thread
 // issues the MMAs and commits them to an mbarrier per stage; all waits are
 // bounded (about 0.1 s of clock cycles) and report a timeout in *err.
-__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t c) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(c) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t par) {
-  uint32_t ok;
-  asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-               : "=r"(ok)
-               : "r"(su32(b)), "r"(par)
-               : "memory");
-  return ok != 0;
-}
-
-// Shared-memory matrix descriptor: 128-byte swizzle, K-major, 1024 B between
-// 8-row groups.
-__device__ __forceinline__ uint64_t sw128_desc(const void* p) {
-  uint64_t d = (su32(p) >> 4) & 0x3FFF;
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;            // descriptor version
-  d |= (uint64_t)2 << 61;            // 128-byte swizzle
-  return d;
-}
-
 __device__ __forceinline__ int sw_off(int r, int c) { return r * 128 + ((c ^ (r & 7)) << 4); }
 
 __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
@@ -646,24 +621,6 @@ __global__ void __launch_bounds__(kThreads) k_gemm_tc(const int32_t* __restrict_
 constexpr int TC2_NRAW = 3;
 constexpr int TC2_RAW = 128 * 128;
 constexpr int TC2_SMEM = TC_STAGE + TC2_NRAW * TC2_RAW + 1024;
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   su32(dst)),
-               "l"(src), "r"(bytes), "r"(su32(b))
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* b, uint32_t par) {
-  const long long t0 = clock64();
-  while (!mbar_try(b, par))
-    if (clock64() - t0 > 200000000LL) return false;
-  return true;
-}
 
 __global__ void __launch_bounds__(kThreads) k_gemm_tc2(const int32_t* __restrict__ blk_sub,
                                                        const int32_t* __restrict__ blk_row0,
