@@ -148,12 +148,14 @@ typedef struct {
                               subdomain (p launches per apply, the plain non-batched form) instead
                               of one batched launch over all subdomains; same results, for
                               measuring what batching buys */
-  int32_t symmetric;       /* FP32 single-vector local applies: 0 = the autotuner picks the
-                              symmetric kernel (reads only the lower block-triangle of F_i / S_i)
-                              when it is faster, 1 = full rows only, 2 = symmetric always
-                              (fastest variant), 3 = symmetric, streamed through shared memory,
-                              4 = symmetric, one CTA per subdomain (transposed partial sums
-                              reduced in shared memory, no second pass) */
+  int32_t symmetric;       /* single-vector local applies: 0 = the autotuner picks the
+                              symmetric kernel (reads only the lower block-triangle of F_i / S_i;
+                              FP64: its 56-bit fixed-point copy) when it is faster, 1 = full rows
+                              only, 2 = symmetric always (fastest variant; FP64 only while an
+                              operator fits the kernel's shared memory), 3 = symmetric, the FP32
+                              one streamed through shared memory, 4 = symmetric, the FP32 one with
+                              one CTA per subdomain (transposed partial sums reduced in shared
+                              memory, no second pass) */
   uint64_t spin_timeout_ns; /* budget of each main-loop mbarrier wait of the streamed symmetric
                                apply and the warp-specialised tensor-core block GEMM, in ns,
                                counted as SM clock cycles at the device's maximum clock
@@ -396,7 +398,9 @@ feti_status feti_element_stats(const feti_ctx* ctx, double* elem_ms, double* ele
 /* Launch schedules of the dense local applies chosen by the setup-time
  * autotuner (timed on the real operators, fastest kept): out[0..1] rows per
  * warp step and rows per CTA of the FP64 F_i apply, out[2..3] of the FP64
- * preconditioner apply, out[4..7] the same for the FP32 copies (rows per warp
+ * preconditioner apply (rows per warp step -400 - C, rows 16 = symmetric
+ * kernel on 56-bit fixed-point panels of 16 rows, C CTAs per subdomain),
+ * out[4..7] the same for the FP32 copies (rows per warp
  * step -G, rows 32 = symmetric kernel on 32-row panels, load groups of
  * G % 100 rows with an L2 prefetch G / 100 tiles ahead; G = 64: panels
  * streamed through shared memory; G = 300 + g: one CTA per subdomain, load

@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libfeti.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["feti_kernels.cu", "feti_kernels_multi.cu", "feti_chol_tc.cu", "feti_factor32.cu", "feti_coarse.cu", "feti_noalloc.cu", "feti_host.cpp",
+SOURCES = ["feti_kernels.cu", "feti_kernels_multi.cu", "feti_chol_tc.cu", "feti_symv_fixed.cu", "feti_factor32.cu", "feti_coarse.cu", "feti_noalloc.cu", "feti_host.cpp",
            "feti_coarse_plan.cpp", "feti_checkpoint.cpp"]
 
 
@@ -42,7 +42,7 @@ def build(verbose_ptxas: bool = False, force: bool = False) -> str:
     """Compile and link; returns the library path.  Rebuilds when sources are newer."""
     os.makedirs(BUILD, exist_ok=True)
     srcs = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(INCLUDE, "feti.h"),
-                                                      os.path.join(CSRC, "feti_internal.h"), os.path.join(CSRC, "feti_tc.cuh")]
+                                                      os.path.join(CSRC, "feti_internal.h"), os.path.join(CSRC, "feti_tc.cuh"), os.path.join(CSRC, "feti_fixed.cuh")]
     if not force and os.path.exists(LIB):
         newest = max(os.path.getmtime(s) for s in srcs)
         if os.path.getmtime(LIB) >= newest:

@@ -188,6 +188,13 @@ struct feti_ctx {
   double elem_ms = 0.0, elem_bytes = 0.0;
   // sizes (elements) of d_A, d_S, d_F, d_F32, d_S32, d_F32s, d_S32s, d_symp
   int64_t op_elems[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  // fixed-point panels and row exponents of the FP64 F_i [0] and
+  // preconditioner block [1] (NULL: not kept), and the CTAs per subdomain the
+  // autotuner picked for their apply (0: the FP64 rows are faster)
+  int64_t fix_elems[2] = {0, 0};
+  int2* d_fix[2] = {nullptr, nullptr};
+  int* d_fixexp[2] = {nullptr, nullptr};
+  int fix64[2] = {0, 0};
   // symmetric FP32 local applies: lower block-triangles, transposed-product
   // partials, work lists, and the load-group size picked by the autotuner
   // per matrix (0: the full-row kernel is used)
@@ -680,6 +687,7 @@ feti_status build_decomposition(feti_ctx* ctx) {
   std::vector<std::vector<int32_t>> dense_ldof(P);  // dense index -> local DOF
   std::vector<std::vector<double>> Rd(P);           // R in dense order, n x k
   int64_t aoff = 0, soff = 0, foff = 0, roff = 0, foff32 = 0, soff32 = 0, fsym = 0, ssym = 0, psym = 0;
+  int64_t ffix = 0, sfix = 0;
   int boff = 0, voff = 0, coff = 0;
   // per subdomain (in parallel): free DOFs, kernel basis, fixing DOFs, dense
   // order, envelope and R in dense order; sizes and offsets after
@@ -869,6 +877,7 @@ feti_status build_decomposition(feti_ctx* ctx) {
     L.aoff = aoff; L.soff = soff; L.foff = foff; L.roff = roff;
     L.foff32 = foff32; L.soff32 = soff32;
     L.fsym32 = fsym; L.ssym32 = ssym; L.psym = psym;
+    L.ffix = ffix; L.sfix = sfix;
     ctx->lay[s] = L;
     const int nb = nbp + k;
     {
@@ -877,6 +886,8 @@ feti_status build_decomposition(feti_ctx* ctx) {
       fsym += PH * PH / 2 * pf * (pf + 1);
       ssym += PH * PH / 2 * ps * (ps + 1);
       psym += PH / 2 * ps * (ps - 1);  // sized for the larger (preconditioner) block
+      ffix += feti::fix_entries(nbp);
+      sfix += feti::fix_entries(nb);
     }
     boff += nb;
     voff += n;
@@ -1392,6 +1403,8 @@ feti_status build_decomposition(feti_ctx* ctx) {
   ctx->op_elems[5] = fsym;
   ctx->op_elems[6] = ctx->opt.precond == FETI_PREC_DIRICHLET ? ssym : 1;
   ctx->op_elems[7] = psym;
+  ctx->fix_elems[0] = ffix;
+  ctx->fix_elems[1] = sfix;
   for (int w = 0; w < 2; ++w) {
     // symmetric-apply work lists: one warp per (subdomain, kSymPH-row panel).
     // Panel I carries I + 1 blocks, so the list runs from the longest panels
@@ -1724,6 +1737,11 @@ feti_status factorize_all(feti_ctx* ctx) {
                             mix ? ctx->d_F32 : nullptr, mix ? ctx->d_F32s : nullptr,
                             ctx->keep_factor ? nullptr : ctx->d_Lc));
   FETI_TRY(check_status(ctx, "local factorization"));
+  for (int w = 0; w < 2; ++w)
+    if (ctx->d_fix[w] && (!ctx->tuned || ctx->fix64[w]))
+      feti::launch_fix_operator(ctx->P, ctx->sym_max_m[w], ctx->d_lay, w, w == 0 ? ctx->d_F : ctx->d_S, ctx->d_fixexp[w],
+                                ctx->d_fix[w], ctx->stream);
+  FETI_CK(cudaGetLastError());
   return FETI_OK;
 }
 
@@ -1859,6 +1877,12 @@ void gemv_apply(feti_ctx* ctx, int which, const int* done, bool f32, const void*
   const void* v = vin ? vin : f32 ? (const void*)ctx->d_vloc32 : (const void*)ctx->d_vloc;
   const float* v32 = static_cast<const float*>(v);
   double* yo = yout ? yout : ctx->d_loc;
+  if (!f32 && ctx->fix64[which]) {
+    (void)feti::launch_symv_fixed(ctx->fix64[which], ctx->P, ctx->d_sym_order[which], ctx->sym_max_m[which],
+                                  ctx->d_lay, which, ctx->d_fix[which], ctx->d_fixexp[which],
+                                  static_cast<const double*>(v), yo, done, ctx->stream);
+    return;
+  }
   if (f32 && ctx->sym32[which] == 64 && !ctx->opt.per_subdomain) {
     feti::launch_symv2_f32(ctx->sym_n[which], ctx->d_sym_sub[which], ctx->d_sym_panel[which], ctx->d_lay, which,
                            which == 0 ? ctx->d_F32s : ctx->d_S32s, v32, yo, ctx->d_symp, ctx->maps,
@@ -1953,7 +1977,7 @@ feti_status autotune_run(feti_ctx* ctx);
 // change the operators), so that a new context on the same mesh and
 // partition skips the timing runs.
 struct TunedPick {
-  int t64[2], r64[2], t32[2], r32[2], sym[2];
+  int t64[2], r64[2], t32[2], r32[2], sym[2], fix[2];
 };
 std::mutex g_tune_mu;
 std::unordered_map<uint64_t, TunedPick> g_tune_cache;
@@ -1973,6 +1997,7 @@ uint64_t tune_signature(const feti_ctx* ctx) {
   add(ctx->opt.precond);
   add(ctx->opt.symmetric);
   add(ctx->opt.per_subdomain);
+  add(ctx->opt.local_form);
   add(ctx->device);
   for (const auto& L : ctx->lay) {
     add(L.n);
@@ -2002,6 +2027,7 @@ feti_status autotune(feti_ctx* ctx) {
         ctx->cfg32[w] = ctx->tab[w][tp.t32[w]];
         ctx->cfg32[w].R = tp.r32[w];
         ctx->sym32[w] = tp.sym[w];
+        ctx->fix64[w] = tp.fix[w];
       }
       ctx->tuned = true;
       return FETI_OK;
@@ -2015,6 +2041,7 @@ feti_status autotune(feti_ctx* ctx) {
     tp.t32[w] = tab_index(ctx, w, ctx->cfg32[w]);
     tp.r32[w] = ctx->cfg32[w].R;
     tp.sym[w] = ctx->sym32[w];
+    tp.fix[w] = ctx->fix64[w];
   }
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune_cache[sig] = tp;
@@ -2054,6 +2081,20 @@ feti_status autotune_run(feti_ctx* ctx) {
           if (ms < best) { best = ms; bestc = c; }
         }
       (f32 ? ctx->cfg32[w] : ctx->cfg64[w]) = bestc;
+      ctx->fix64[w] = f32 ? ctx->fix64[w] : 0;
+      if (!f32 && ctx->d_fix[w] && ctx->opt.symmetric >= 2) best = 1e30f;  // always symmetric
+      for (int C = 1; !f32 && ctx->d_fix[w] && C <= 8; C *= 2) {  // fixed-point symmetric form, C CTAs per subdomain
+        float ms = 0.f;
+        for (int rep = -1; rep < 3; ++rep) {
+          if (rep == 0) FETI_CK(cudaEventRecord(e0, st));
+          FETI_CK(feti::launch_symv_fixed(C, ctx->P, ctx->d_sym_order[w], ctx->sym_max_m[w], ctx->d_lay, w, ctx->d_fix[w],
+                                          ctx->d_fixexp[w], ctx->d_vloc, ctx->d_loc, ctx->d_zero, st));
+        }
+        FETI_CK(cudaEventRecord(e1, st));
+        FETI_CK(cudaEventSynchronize(e1));
+        FETI_CK(cudaEventElapsedTime(&ms, e0, e1));
+        if (ms < best) { best = ms; ctx->fix64[w] = C; }
+      }
       if (f32 && ctx->d_F32s && !ctx->opt.per_subdomain) {  // the plain form launches full rows
         // symmetric lower block-triangle kernel: load groups of 8 / 16 / 32 rows,
         // + 100 x (tiles of L2 prefetch ahead)
@@ -2214,6 +2255,16 @@ feti_status alloc_operators(feti_ctx* ctx) {
       FETI_TRY(dev_alloc(ctx, &ctx->d_kzb64, (size_t)ctx->nb_total));
       FETI_TRY(dev_alloc(ctx, &ctx->d_kxb, (size_t)ctx->nb_total));
     }
+  }
+  // fixed-point copies where the FP64 operators are applied in every
+  // iteration or residual: F_i, and S_i in the FP64 form
+  for (int w = 0; w < 2; ++w) {
+    if (!fp64_ops(ctx) || ctx->opt.per_subdomain || ctx->opt.symmetric == 1 || ctx->sym_max_m[w] <= 0 ||
+        !feti::symv_fixed_fits(ctx->sym_max_m[w]))
+      continue;
+    if (w == 0 ? ctx->opt.local_form == 2 : ctx->opt.precond != FETI_PREC_DIRICHLET || f32_ops(ctx)) continue;
+    FETI_TRY(dev_alloc(ctx, &ctx->d_fix[w], (size_t)ctx->fix_elems[w]));
+    FETI_TRY(dev_alloc(ctx, &ctx->d_fixexp[w], (size_t)ctx->nb_total));
   }
   if (f32_ops(ctx)) {
     FETI_TRY(dev_alloc(ctx, &ctx->d_F32, (size_t)ctx->op_elems[3]));
@@ -3582,8 +3633,8 @@ feti_status feti_get_schedule(const feti_ctx* ctx, int32_t out[12]) {
   if (!ctx || !out) return FETI_ERR_INVALID_ARG;
   for (int i = 8; i < 12; ++i) out[i] = -1;
   for (int w = 0; w < 2; ++w) {
-    out[2 * w] = ctx->cfg64[w].R;
-    out[2 * w + 1] = ctx->cfg64[w].rpc;
+    out[2 * w] = ctx->fix64[w] ? -400 - ctx->fix64[w] : ctx->cfg64[w].R;
+    out[2 * w + 1] = ctx->fix64[w] ? feti::kFixRows : ctx->cfg64[w].rpc;
     out[4 + 2 * w] = ctx->sym32[w] ? -ctx->sym32[w] : ctx->cfg32[w].R;
     out[4 + 2 * w + 1] = ctx->sym32[w] ? feti::kSymPH : ctx->cfg32[w].rpc;
     if (ctx->tuned_m) {

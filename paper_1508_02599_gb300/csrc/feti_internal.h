@@ -47,11 +47,16 @@ struct SubLayout {
   int64_t psym;   // offset (floats) of the transposed-product partials: PH I floats per panel I
   int64_t loff;   // offset of the compact interior factor: rows [0, nI + nbp) x columns [0, nI)
                   // of the Cholesky factor (L_II lower, L_bI), row stride kp_ld
+  // 56-bit fixed-point panels of the FP64 F_i and preconditioner block
+  // (entries): kFixRows-row panels of the lower block triangle
+  int64_t ffix;
+  int64_t sfix;
   int64_t zoff;   // offset (bytes) of the elimination scratch, relative to the group's first
 };
 // Row stride of the compact interior factor (a multiple of 4 elements).
 __host__ __device__ inline int kp_ld(const SubLayout& L) { return (L.nI + 3) & ~3; }
 constexpr int kSymPH = 32;  // panel height of the symmetric FP32 apply
+constexpr int kFixRows = 16;  // panel height of the fixed-point symmetric FP64 apply
 
 // Element kernels ------------------------------------------------------------
 // Element matrices are symmetric and stored as their upper triangle, row by
@@ -204,6 +209,20 @@ void launch_symv2_f32(int n_warps, const int32_t* wsub, const int32_t* wpanel, c
 // pass; max_m: the largest operator size.  G = 8, 16 or 32.
 void launch_symv3_f32(int G, int P, const int32_t* order, int max_m, const SubLayout* lay, int which,
                       const float* Msym, const float* vloc, double* y, const int* done, cudaStream_t st);
+// FP64 apply of F_i (which 0) or the preconditioner block (which 1) from the
+// lower block triangle in 56-bit fixed point (feti_symv_fixed.cu).
+// launch_fix_operator: row exponents (ex, boundary offsets) and panels out of
+// the full FP64 matrices; launch_symv_fixed: y = M v with C CTAs per
+// subdomain (1, 2, 4 or 8), order: subdomains largest first;
+// fix_entries: entries of the panels of an operator of m rows;
+// symv_fixed_fits: whether operators up to max_m rows can be applied.
+int64_t fix_entries(int m);
+bool symv_fixed_fits(int max_m);
+void launch_fix_operator(int P, int max_m, const SubLayout* lay, int which, const double* M, int* ex, int2* out,
+                         cudaStream_t st);
+cudaError_t launch_symv_fixed(int C, int P, const int32_t* order, int max_m, const SubLayout* lay, int which,
+                              const int2* M, const int* ex, const double* vloc, double* y, const int* done,
+                              cudaStream_t st);
 // FP32 signed gather (input of the FP32 apply).
 void launch_gather32(const Maps& mp, const double* x, const double* wv, float* y, const int* done, cudaStream_t st);
 // a += b
