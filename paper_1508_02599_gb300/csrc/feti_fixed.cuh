@@ -14,6 +14,13 @@ __device__ __forceinline__ long long shift_even(unsigned long long q, int r) {
   return (long long)((q + (((1ull << r) - 1) >> 1) + ((q >> r) & 1)) >> r);
 }
 
+// a b + c as one instruction (the compiler's own form of the expression takes
+// one and a half, 28 against 46 lanes per clock and SM)
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+  return c;
+}
+
 // biased exponent of an FP64 number (0: zero or subnormal, 2047: not finite)
 __device__ __forceinline__ int bexp64(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 

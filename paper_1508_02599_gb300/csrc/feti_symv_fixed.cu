@@ -96,13 +96,6 @@ __global__ void __launch_bounds__(256) k_fix_pack(const SubLayout* __restrict__ 
   }
 }
 
-// a b + c as one instruction (the compiler's own form of the expression takes
-// one and a half, 28 against 46 lanes per clock and SM)
-__device__ __forceinline__ long long mad(int a, int b, long long c) {
-  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
-  return c;
-}
-
 // A warp's place in its panels: panel of rows r0 .. and w columns, tile at
 // column c0, the lane's two entries of its first row at p.
 struct Place {
@@ -140,29 +133,29 @@ __device__ __forceinline__ void mul_group(const int4 (&a)[GR], const int2* __res
 #pragma unroll
   for (int r = 0; r < GR; r += 4) {  // four rows at a time: independent accumulators side by side
 #pragma unroll
-    for (int i = r; i < r + 4; ++i) rh[i] = mad(a[i].x, vc.x, rh[i]);
+    for (int i = r; i < r + 4; ++i) rh[i] = mad_wide(a[i].x, vc.x, rh[i]);
 #pragma unroll
-    for (int i = r; i < r + 4; ++i) rc[i] = mad(a[i].x, vc.y, rc[i]);
+    for (int i = r; i < r + 4; ++i) rc[i] = mad_wide(a[i].x, vc.y, rc[i]);
     int2 v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = vr[r + i];
 #pragma unroll
-    for (int i = r; i < r + 4; ++i) rh[i] = mad(a[i].z, vc.z, rh[i]);
+    for (int i = r; i < r + 4; ++i) rh[i] = mad_wide(a[i].z, vc.z, rh[i]);
 #pragma unroll
-    for (int i = r; i < r + 4; ++i) rc[i] = mad(a[i].y, vc.x, rc[i]);
+    for (int i = r; i < r + 4; ++i) rc[i] = mad_wide(a[i].y, vc.x, rc[i]);
 #pragma unroll
     for (int i = r; i < r + 4; ++i) {
-      col[0] = mad(a[i].x, v[i - r].x, col[0]);
-      col[1] = mad(a[i].x, v[i - r].y, col[1]);
-      col[2] = mad(a[i].z, v[i - r].x, col[2]);
-      col[3] = mad(a[i].z, v[i - r].y, col[3]);
-      rc[i] = mad(a[i].z, vc.w, rc[i]);
+      col[0] = mad_wide(a[i].x, v[i - r].x, col[0]);
+      col[1] = mad_wide(a[i].x, v[i - r].y, col[1]);
+      col[2] = mad_wide(a[i].z, v[i - r].x, col[2]);
+      col[3] = mad_wide(a[i].z, v[i - r].y, col[3]);
+      rc[i] = mad_wide(a[i].z, vc.w, rc[i]);
     }
 #pragma unroll
     for (int i = r; i < r + 4; ++i) {
-      rc[i] = mad(a[i].w, vc.z, rc[i]);
-      col[1] = mad(a[i].y, v[i - r].x, col[1]);
-      col[3] = mad(a[i].w, v[i - r].x, col[3]);
+      rc[i] = mad_wide(a[i].w, vc.z, rc[i]);
+      col[1] = mad_wide(a[i].y, v[i - r].x, col[1]);
+      col[3] = mad_wide(a[i].w, v[i - r].x, col[3]);
     }
   }
 }
