@@ -78,8 +78,8 @@ void launch_elem_hgo(int n_tets, const double* coords, const int32_t* tets, cons
 // p0: volumetric part condensed to a piecewise-constant pressure (P2-P0).
 void launch_elem_linear_p2(int n_tets, const double* coords, const int32_t* tets, double E, double nu, int p0,
                            double* Ke, int* status, cudaStream_t st);
-// Local assembly: one CTA per subdomain walks its elements in order (no
-// atomics); nde = DOFs per element (12 for P1, 30 for P2), Ke stride nde^2.
+// Local assembly: the warps of a subdomain own its rows and scan its elements
+// in order (no atomics); nde = DOFs per element (12 for P1, 30 for P2), Ke stride nde^2.
 void launch_assemble(int P, const SubLayout* lay, const int32_t* sub_elem_ptr, const int32_t* sub_elems,
                      const int32_t* elem_dense, const double* Ke, int nde, double* A, cudaStream_t st);
 // Local load vectors: surface loads (+ -f_int) (- K_iD u_D); fdn = DOFs per

@@ -362,35 +362,66 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
 }
 
 // ---------------------------------------------------------------------------
+// Local assembly without atomics: 64 warps per subdomain (eight CTAs), each the
+// owner of the local rows r with r mod 64 equal to its number.  A warp scans
+// the subdomain's elements in order and adds only the element rows it owns, so
+// every entry is summed in element order whatever runs beside it.  The scan
+// reads 48 bytes an element (from the second-level cache for all but one owner)
+// and the chain of additions of one CTA per subdomain that walked the elements
+// one by one, 3 us each, is split 64 ways: 16.0 -> 1.0 ms on the 1024-subdomain
+// tube, 4.8 -> 0.1 ms on the 64-subdomain one.
+constexpr int kOwners = 64;
+constexpr int kOwnerCtas = kOwners / (kThreads / 32);
+
+// Element rows of the elements q .. of a subdomain, 16 (nde <= 16) or 32 lanes
+// per element; f(e, il, r, base) for every owned one in element order: element,
+// local row, matrix row and first lane of the element's rows (all lanes call it).
+template <typename F>
+__device__ __forceinline__ void owned_rows(int q0, int q1, const int32_t* __restrict__ list,
+                                           const int32_t* __restrict__ dense, int nde, int owner, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const int wd = nde <= 16 ? 16 : 32, per = 32 / wd;
+  const int i = lane & (wd - 1), sub = lane / wd;
+  for (int q = q0; q < q1; q += 4 * per) {
+    int e[4], r[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = q + u * per + sub;
+      e[u] = k < q1 ? (list ? list[k] : k) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) r[u] = e[u] >= 0 && i < nde ? dense[(size_t)nde * e[u] + i] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      unsigned mask = __ballot_sync(0xffffffffu, r[u] >= 0 && (r[u] & (kOwners - 1)) == owner);
+      while (mask) {
+        const int src = __ffs(mask) - 1;
+        mask &= mask - 1;
+        f(__shfl_sync(0xffffffffu, e[u], src), src & (wd - 1), r[u], src);
+        __syncwarp();  // an entry's next addition may come from another lane
+      }
+    }
+  }
+}
+
 // T = double (FP64 factorization) or float (FP32 factorization: each entry
 // is summed in FP32 in element order).
 template <typename T>
-__global__ void k_assemble(const SubLayout* __restrict__ lay, const int32_t* __restrict__ sub_elem_ptr,
-                           const int32_t* __restrict__ sub_elems, const int32_t* __restrict__ elem_dense,
-                           const double* __restrict__ Ke, int nde, T* __restrict__ Abase) {
-  const int s = blockIdx.x;
+__global__ void __launch_bounds__(kThreads) k_assemble(const SubLayout* __restrict__ lay,
+                                                       const int32_t* __restrict__ sub_elem_ptr,
+                                                       const int32_t* __restrict__ sub_elems,
+                                                       const int32_t* __restrict__ elem_dense,
+                                                       const double* __restrict__ Ke, int nde, T* __restrict__ Abase) {
+  const int s = blockIdx.y;
   const SubLayout L = lay[s];
   T* A = Abase + L.aoff;
   const int kes = ke_packed(nde);
-  for (int q = sub_elem_ptr[s]; q < sub_elem_ptr[s + 1]; ++q) {
-    const int e = sub_elems[q];
-    for (int t = threadIdx.x; t < kes; t += blockDim.x) {
-      // packed entry t -> (i, j), i <= j; both (i, j) and (j, i) of the local matrix
-      int i = 0, rem = t;
-      while (rem >= nde - i) {
-        rem -= nde - i;
-        ++i;
-      }
-      const int j = i + rem;
-      const int r = elem_dense[(size_t)nde * e + i], c = elem_dense[(size_t)nde * e + j];
-      if (r >= 0 && c >= 0) {
-        const T v = (T)Ke[(size_t)e * kes + t];
-        A[(size_t)r * L.ld + c] += v;
-        if (i != j) A[(size_t)c * L.ld + r] += v;
-      }
-    }
-    __syncthreads();
-  }
+  const int lane = threadIdx.x & 31, owner = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  owned_rows(sub_elem_ptr[s], sub_elem_ptr[s + 1], sub_elems, elem_dense, nde, owner, [&](int e, int il, int r, int src) {
+    const int row = __shfl_sync(0xffffffffu, r, src);
+    const int c = __shfl_sync(0xffffffffu, r, src - il + (lane < nde ? lane : 0));
+    if (lane < nde && c >= 0) A[(size_t)row * L.ld + c] += (T)Ke[(size_t)e * kes + ke_idx(nde, il, lane)];
+  });
 }
 
 // Consistent nodal loads of one loaded face under constant pressure (kind 0,
@@ -428,43 +459,41 @@ __global__ void k_face_forces(int n_faces, int fpn, const int32_t* __restrict__ 
       out[3 * (size_t)fpn * f + 3 * v + i] = (fpn == 3 || v >= 3) ? force[i] : 0.0;
 }
 
-__global__ void k_assemble_rhs(const SubLayout* __restrict__ lay, const int32_t* __restrict__ sub_face_ptr,
-                               const int32_t* __restrict__ face_dense, const double* __restrict__ face_force, int fdn,
-                               const int32_t* __restrict__ sub_elem_ptr, const int32_t* __restrict__ sub_elems,
-                               const int32_t* __restrict__ elem_dense, const double* __restrict__ elem_dirval,
-                               const double* __restrict__ Ke, const double* __restrict__ fe, int nde, double tau,
-                               double* __restrict__ fbase) {
-  const int s = blockIdx.x;
+// Local load vectors by the same owners: zero, the loaded faces, then the
+// elements (-f_int, and -K_iD u_D of eliminated Dirichlet DOFs), each row in
+// that order.
+__global__ void __launch_bounds__(kThreads) k_assemble_rhs(
+    const SubLayout* __restrict__ lay, const int32_t* __restrict__ sub_face_ptr, const int32_t* __restrict__ face_dense,
+    const double* __restrict__ face_force, int fdn, const int32_t* __restrict__ sub_elem_ptr,
+    const int32_t* __restrict__ sub_elems, const int32_t* __restrict__ elem_dense,
+    const double* __restrict__ elem_dirval, const double* __restrict__ Ke, const double* __restrict__ fe, int nde,
+    double tau, double* __restrict__ fbase) {
+  const int s = blockIdx.y;
   const SubLayout L = lay[s];
   double* f = fbase + L.voff;
-  const int t = threadIdx.x;
-  for (int i = t; i < L.n; i += blockDim.x) f[i] = 0.0;
-  __syncthreads();
-  for (int q = sub_face_ptr[s]; q < sub_face_ptr[s + 1]; ++q) {
-    if (t < fdn) {
-      const int r = face_dense[(size_t)fdn * q + t];
-      if (r >= 0) f[r] += tau * face_force[(size_t)fdn * q + t];
-    }
-    __syncthreads();
-  }
+  const int lane = threadIdx.x & 31, owner = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  for (int r = owner + kOwners * lane; r < L.n; r += 32 * kOwners) f[r] = 0.0;
+  __syncwarp();
+  owned_rows(sub_face_ptr[s], sub_face_ptr[s + 1], nullptr, face_dense, fdn, owner, [&](int q, int il, int r, int src) {
+    if (lane == src) f[r] += tau * face_force[(size_t)fdn * q + il];
+  });
+  if (!fe && !elem_dirval) return;
   const int kes = ke_packed(nde);
-  for (int q = sub_elem_ptr[s]; q < sub_elem_ptr[s + 1]; ++q) {
-    const int e = sub_elems[q];
-    if (t < nde) {
-      const int r = elem_dense[(size_t)nde * e + t];
-      if (r >= 0) {
-        double v = fe ? -fe[(size_t)e * nde + t] : 0.0;
-        if (elem_dirval) {
-          for (int b = 0; b < nde; ++b) {
-            const double ud = elem_dirval[(size_t)nde * e + b];
-            if (ud != 0.0) v -= Ke[(size_t)e * kes + ke_idx(nde, t, b)] * ud;
-          }
+  owned_rows(sub_elem_ptr[s], sub_elem_ptr[s + 1], sub_elems, elem_dense, nde, owner, [&](int e, int il, int r, int src) {
+    double v = fe ? -fe[(size_t)e * nde + il] : 0.0;
+    if (elem_dirval) {
+      const double ud = lane < nde ? elem_dirval[(size_t)nde * e + lane] : 0.0;
+      unsigned on = __ballot_sync(0xffffffffu, ud != 0.0);
+      if (on) {
+        const double k = lane < nde ? Ke[(size_t)e * kes + ke_idx(nde, il, lane)] : 0.0;
+        for (; on; on &= on - 1) {
+          const int b = __ffs(on) - 1;
+          v -= __shfl_sync(0xffffffffu, k, b) * __shfl_sync(0xffffffffu, ud, b);
         }
-        f[r] += v;
       }
     }
-    __syncthreads();
-  }
+    if (lane == src && v != 0.0) f[r] += v;
+  });
 }
 
 template <typename T>
@@ -1516,19 +1545,19 @@ void launch_elem_hgo(int n_tets, const double* coords, const int32_t* tets, cons
 
 void launch_assemble(int P, const SubLayout* lay, const int32_t* sub_elem_ptr, const int32_t* sub_elems,
                      const int32_t* elem_dense, const double* Ke, int nde, double* A, cudaStream_t st) {
-  k_assemble<double><<<P, nde > 12 ? 256 : 160, 0, st>>>(lay, sub_elem_ptr, sub_elems, elem_dense, Ke, nde, A);
+  k_assemble<double><<<dim3(kOwnerCtas, P), kThreads, 0, st>>>(lay, sub_elem_ptr, sub_elems, elem_dense, Ke, nde, A);
 }
 
 void launch_assemble(int P, const SubLayout* lay, const int32_t* sub_elem_ptr, const int32_t* sub_elems,
                      const int32_t* elem_dense, const double* Ke, int nde, float* A, cudaStream_t st) {
-  k_assemble<float><<<P, nde > 12 ? 256 : 160, 0, st>>>(lay, sub_elem_ptr, sub_elems, elem_dense, Ke, nde, A);
+  k_assemble<float><<<dim3(kOwnerCtas, P), kThreads, 0, st>>>(lay, sub_elem_ptr, sub_elems, elem_dense, Ke, nde, A);
 }
 
 void launch_assemble_rhs(int P, const SubLayout* lay, const int32_t* sub_face_ptr, const int32_t* face_dense,
                          const double* face_force, int fdn, const int32_t* sub_elem_ptr, const int32_t* sub_elems,
                          const int32_t* elem_dense, const double* elem_dirval, const double* Ke, const double* fe,
                          int nde, double tau, double* f, cudaStream_t st) {
-  k_assemble_rhs<<<P, 128, 0, st>>>(lay, sub_face_ptr, face_dense, face_force, fdn, sub_elem_ptr, sub_elems,
+  k_assemble_rhs<<<dim3(kOwnerCtas, P), kThreads, 0, st>>>(lay, sub_face_ptr, face_dense, face_force, fdn, sub_elem_ptr, sub_elems,
                                      elem_dense, elem_dirval, Ke, fe, nde, tau, f);
 }
 
