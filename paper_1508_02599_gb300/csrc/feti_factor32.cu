@@ -80,10 +80,10 @@ __global__ void __launch_bounds__(256) k_extract_tiles(const SubLayout* __restri
 //   y_I = L_II^-1 r_I,   z_b = r_b - L_bI y_I,   x_b = (L_bb L_bb^T)^-1 z_b = F_i z_b,
 //   x_I = L_II^-T (y_I - L_bI^T x_b),
 // and F_i = S_i[b',b']^-1 is the explicit FP32 operator the PCG already
-// applies.  The dependent 32-row block chains shrink from n_I + n_b' rows to
+// applies.  The dependent 64-row block chains shrink from n_I + n_b' rows to
 // n_I rows; the boundary panel products carry no chain.
 // The sweeps in four kernels: the two triangular chains over L_II run one
-// CTA per subdomain (k_kp_fwd_interior, k_kp_bwd_interior: 32-row blocks one
+// CTA per subdomain (k_kp_fwd_interior, k_kp_bwd_interior: 64-row blocks one
 // after another), and the two products with L_bI, which carry no chain and
 // hold most of the factor's bytes, run many CTAs per subdomain
 // (k_kp_fwd_boundary: 32 boundary rows per CTA; k_kp_bwd_boundary: 32
@@ -96,94 +96,92 @@ __device__ __forceinline__ T kp_warp_sum(T v) {
   return v;
 }
 
-// Diagonal block [I0, I0 + 32) of L_II (lower triangle, zero elsewhere) into D.
-template <typename T>
-__device__ __forceinline__ void kp_load_diag(const T* __restrict__ A, size_t ld, int nI, int I0, T (*D)[33]) {
-  const int nb = min(32, nI - I0);
-  for (int idx = threadIdx.x; idx < 32 * 32; idx += kT) {
-    const int rr = idx >> 5, c = idx & 31;
-    D[rr][c] = (rr < nb && c <= rr) ? A[(size_t)(I0 + rr) * ld + I0 + c] : (T)0;
-  }
-}
+// The diagonal blocks of the compact factor are stored inverted: rows and
+// columns [64 b, 64 b + 64) of L_II hold W_b = L_bb^-1 (k_tcc_diag), so a block's
+// solve is a product over all threads.  A substitution by one warp costs a
+// division and a product in a row for each of its columns, every one of them
+// some 65 clocks of issue in FP64: 27 us per 32 columns, 0.55 ms for the 640
+// interior DOFs of a sub-cube, where the whole sweep is 0.05 ms of FP64 issue.
+constexpr int kKB = kCholPanel;  // block of the sweeps
 
-// ys[i] -= L[i, I0 : I0 + 32] . xs for the rows i in [i0, nI), a thread per
-// row, the 32 entries read as 16-byte vectors (rows and I0 are multiples of 4
-// elements apart from an aligned base).
-__device__ __forceinline__ void kp_row_update(const float* __restrict__ A, size_t ld, int I0, int i0, int nI,
-                                              const float* xs, float* ys) {
-  // two halves of 16 entries: the FP32 sweeps run 8 CTAs of 256 threads per
-  // SM (one wave over a thousand subdomains), 32 registers a thread
-  for (int i = i0 + threadIdx.x; i < nI; i += kT) {
-    const float4* row = reinterpret_cast<const float4*>(A + (size_t)i * ld + I0);
-    float acc = 0.0f;
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      float4 a[4];
+// Sixteen consecutive entries at p (16-byte aligned), the first n of them.
+__device__ __forceinline__ void load16(const float* __restrict__ p, int n, float (&a)[16]) {
+  if (n >= 16) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = __ldg(row + 4 * h + u);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float* xv = xs + 16 * h + 4 * u;
-        acc += a[u].x * xv[0] + a[u].y * xv[1] + a[u].z * xv[2] + a[u].w * xv[3];
-      }
+    for (int u = 0; u < 4; ++u) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(p) + u);
+      a[4 * u] = v.x, a[4 * u + 1] = v.y, a[4 * u + 2] = v.z, a[4 * u + 3] = v.w;
     }
-    ys[i] -= acc;
+  } else {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) a[u] = u < n ? __ldg(p + u) : 0.0f;
   }
 }
-__device__ __forceinline__ void kp_row_update(const double* __restrict__ A, size_t ld, int I0, int i0, int nI,
-                                              const double* xs, double* ys) {
-  for (int i = i0 + threadIdx.x; i < nI; i += kT) {
-    const double2* row = reinterpret_cast<const double2*>(A + (size_t)i * ld + I0);
-    double2 a[16];
+__device__ __forceinline__ void load16(const double* __restrict__ p, int n, double (&a)[16]) {
+  if (n >= 16) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) a[u] = __ldg(row + u);
-    double acc = 0.0;
+    for (int u = 0; u < 8; ++u) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(p) + u);
+      a[2 * u] = v.x, a[2 * u + 1] = v.y;
+    }
+  } else {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) acc += a[u].x * xs[2 * u] + a[u].y * xs[2 * u + 1];
-    ys[i] -= acc;
+    for (int u = 0; u < 16; ++u) a[u] = u < n ? __ldg(p + u) : 0.0;
   }
+}
+// sum over the four lanes of a row
+template <typename T>
+__device__ __forceinline__ T quad_sum(T v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
 // y_I = L_II^-1 r_I (into yI at the subdomain's local offset), right-looking
-// by 32-column blocks: warp 0 solves the diagonal block, then every thread
-// updates the rows below it with the block's 32 solved values while the next
-// diagonal block is fetched into the other buffer.
+// by 64-column blocks, four threads per row (16 columns each): y_b = W_b r_b,
+// then the rows below are updated with it.  The next block's W and the first
+// rows to update are fetched before they are needed.
 template <typename T>
-__global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 8 : 4)
+__global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
     k_kp_fwd_interior(const SubLayout* __restrict__ lay, const T* __restrict__ Lbase, const double* __restrict__ rbase,
                       T* __restrict__ yIbase) {
   extern __shared__ __align__(16) unsigned char kp_smem[];
-  T* ys = reinterpret_cast<T*>(kp_smem);
+  T* ys = reinterpret_cast<T*>(kp_smem);  // [nI rounded up to 64], zero beyond nI
   const SubLayout L = lay[blockIdx.x];
   const T* A = Lbase + L.loff;
   const size_t ld = kp_ld(L);
   const double* r = rbase + L.voff;
   const int nI = L.nI;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ T Db[2][32][33];
-  __shared__ __align__(16) T xs[32];
-  for (int i = tid; i < nI; i += kT) ys[i] = (T)r[i];
-  if (nI > 0) kp_load_diag(A, ld, nI, 0, Db[0]);
+  const int tid = threadIdx.x, row = tid >> 2, c = 16 * (tid & 3);
+  T w[16], a[16];
+  // entries [row i, columns I0 + c ..), the columns up to `end`
+  auto fetch = [&](T (&v)[16], int i, int I0, int end) {
+    load16(A + (size_t)min(i, nI - 1) * ld + I0 + c, i < nI ? end - I0 - c : 0, v);
+  };
+  if (nI > 0) fetch(w, row, 0, nI);
+  for (int i = tid; i < (nI + kKB - 1) / kKB * kKB; i += kT) ys[i] = i < nI ? (T)r[i] : (T)0;
   __syncthreads();
-  for (int I0 = 0, k = 0; I0 < nI; I0 += 32, ++k) {
-    const int nb = min(32, nI - I0);
-    T (*D)[33] = Db[k & 1];
-    if (warp == 0) {
-      T b = lane < nb ? ys[I0 + lane] : (T)0;
-      T xv = 0;
-      for (int c = 0; c < nb; ++c) {
-        if (lane == c) xv = b / D[c][c];
-        const T xc = __shfl_sync(0xffffffffu, xv, c);
-        if (lane > c) b -= D[lane][c] * xc;
-      }
-      if (lane < nb) ys[I0 + lane] = xv;
-      xs[lane] = lane < nb ? xv : (T)0;
-    }
+  for (int I0 = 0; I0 < nI; I0 += kKB) {
+    const int I1 = I0 + kKB;
+    T acc = 0;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) acc += w[u] * ys[I0 + c + u];
+    acc = quad_sum(acc);
+    const bool more = I1 < nI;  // then the block is whole
+    if (more) fetch(a, I1 + row, I0, I1);
     __syncthreads();
-    const int I1 = I0 + 32;
-    if (I1 < nI) {  // then nb == 32
-      kp_load_diag(A, ld, nI, I1, Db[(k + 1) & 1]);
-      kp_row_update(A, ld, I0, I1, nI, xs, ys);
+    if (c == 0) ys[I0 + row] = acc;  // rows beyond nI: zero
+    if (more) fetch(w, I1 + row, I1, nI);
+    __syncthreads();
+    if (!more) break;
+    const T* xs = ys + I0 + c;
+    for (int i = I1 + row;; i += kKB) {
+      T t = 0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) t += a[u] * xs[u];
+      t = quad_sum(t);
+      if (c == 0 && i < nI) ys[i] -= t;
+      if (i - row + kKB >= nI) break;
+      fetch(a, i + kKB, I0, I1);
     }
     __syncthreads();
   }
@@ -288,17 +286,17 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 8 : 4)
   }
 }
 
-// x_I = L_II^-T t_I (t_I in yI after k_kp_bwd_boundary), by 32-column
-// blocks from the last: warp 0 solves the transposed diagonal block, then a
-// thread per column j below the block's start subtracts L[I0 : I0 + 32, j]^T
-// times the block's solved values (32 loads in flight per thread) while the
-// previous diagonal block is fetched into the other buffer; then x (+)= x on
-// rows [0, n_I + n_b') (x_b from the F_i apply, FP64 at the boundary offset),
-// and with init x = that correction, zero on the fixing rows.
+// x_I = L_II^-T t_I (t_I in yI after k_kp_bwd_boundary), by 64-column blocks
+// from the last: x_b = W_b^T t_b, then L[b, j]^T x_b is taken from every column j
+// before the block; then x (+)= x on rows [0, n_I + n_b') (x_b from the F_i
+// apply, FP64 at the boundary offset), and with init x = that correction,
+// zero on the fixing rows.  `parts` threads share a column (4, or 1 where the
+// copies do not fit), each with 64 / parts of a block's rows and its own copy of
+// the subtracted sums, added in a fixed order when the block is reached.
 template <typename T>
-__global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 8 : 4)
+__global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
     k_kp_bwd_interior(const SubLayout* __restrict__ lay, const T* __restrict__ Lbase, const T* __restrict__ yIbase,
-                      const double* __restrict__ xb, double* __restrict__ xbase, int init) {
+                      const double* __restrict__ xb, double* __restrict__ xbase, int init, int parts) {
   extern __shared__ __align__(16) unsigned char kp_smem[];
   T* ys = reinterpret_cast<T*>(kp_smem);
   const SubLayout L = lay[blockIdx.x];
@@ -306,47 +304,52 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 8 : 4)
   const size_t ld = kp_ld(L);
   double* x = xbase + L.voff;
   const int nI = L.nI, nbp = L.nbp;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ T Db[2][32][33];
-  __shared__ T xs[32];
+  const int nIp = (nI + kKB - 1) / kKB * kKB;
+  T* sub = ys + nIp;  // [parts][nIp]
+  const int tid = threadIdx.x;
+  __shared__ T ts[kKB], ps[4][kKB];
+  const int wj = tid & 63, wi = 16 * (tid >> 6);
+  T w[16];
+  auto fetch_w = [&](int I0) {  // rows wi .., column wj of W_b
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = I0 + wi + u;
+      w[u] = (i < nI && wj <= wi + u) ? __ldg(A + (size_t)i * ld + I0 + wj) : (T)0;
+    }
+  };
+  if (nI > 0) fetch_w(nIp - kKB);
   const T* yI = yIbase + L.voff;
-  for (int i = tid; i < nI; i += kT) ys[i] = yI[i];
-  const int Ilast = nI > 0 ? ((nI - 1) / 32) * 32 : -32;
-  if (Ilast >= 0) kp_load_diag(A, ld, nI, Ilast, Db[0]);
+  for (int i = tid; i < nIp; i += kT) ys[i] = i < nI ? yI[i] : (T)0;
+  for (int i = tid; i < parts * nIp; i += kT) sub[i] = (T)0;
   __syncthreads();
-  for (int I0 = Ilast, k = 0; I0 >= 0; I0 -= 32, ++k) {
-    const int nb = min(32, nI - I0);
-    T (*D)[33] = Db[k & 1];
-    if (warp == 0) {
-      T b = lane < nb ? ys[I0 + lane] : (T)0;
-      T xv = 0;
-      for (int c = nb - 1; c >= 0; --c) {
-        if (lane == c) xv = b / D[c][c];
-        const T xc = __shfl_sync(0xffffffffu, xv, c);
-        if (lane < c) b -= D[c][lane] * xc;
-      }
-      if (lane < nb) ys[I0 + lane] = xv;
-      xs[lane] = lane < nb ? xv : (T)0;
+  const int per = kT / parts, col = tid % per, rows = kKB / parts, i0 = (tid / per) * rows;
+  T* mine = sub + (size_t)(tid / per) * nIp;
+  for (int I0 = nIp - kKB; I0 >= 0; I0 -= kKB) {
+    if (tid < kKB) {
+      T t = ys[I0 + tid];
+      for (int k = 0; k < parts; ++k) t -= sub[(size_t)k * nIp + I0 + tid];
+      ts[tid] = t;
     }
     __syncthreads();
-    if (I0 > 0) {
-      kp_load_diag(A, ld, nI, I0 - 32, Db[(k + 1) & 1]);
-      const T* blk = A + (size_t)I0 * ld;
-      for (int j = tid; j < I0; j += kT) {
-        T acc = 0;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          T a[16];
+    T acc = 0;
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            const int rr = 16 * h + u;
-            a[u] = rr < nb ? __ldg(blk + (size_t)rr * ld + j) : (T)0;
-          }
+    for (int u = 0; u < 16; ++u) acc += w[u] * ts[wi + u];
+    ps[tid >> 6][wj] = acc;
+    if (I0 > 0) fetch_w(I0 - kKB);
+    __syncthreads();
+    if (tid < kKB) ys[I0 + tid] = (ps[0][tid] + ps[1][tid]) + (ps[2][tid] + ps[3][tid]);
+    __syncthreads();
+    const T* blk = A + (size_t)I0 * ld;
+    for (int j = col; j < I0; j += per) {
+      T t = 0;
+      for (int h = i0; h < i0 + rows; h += 16) {
+        T a[16];
 #pragma unroll
-          for (int u = 0; u < 16; ++u) acc += a[u] * xs[16 * h + u];
-        }
-        ys[j] -= acc;
+        for (int u = 0; u < 16; ++u) a[u] = I0 + h + u < nI ? __ldg(blk + (size_t)(h + u) * ld + j) : (T)0;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) t += a[u] * ys[I0 + h + u];
       }
+      mine[j] += t;
     }
     __syncthreads();
   }
@@ -503,46 +506,49 @@ void kp_smem_attr(K kern, size_t smem) {
 }
 
 template <typename T>
-void kp_forward(int P, const SubLayout* lay, const T* Lc, const double* r, T* yI, T* zb, int max_nr, cudaStream_t st) {
+void kp_forward(int P, const SubLayout* lay, const T* Lc, const double* r, T* yI, T* zb, int max_nr, int max_nI, cudaStream_t st) {
   if (P <= 0) return;
   const size_t smem = (size_t)std::max(max_nr, 1) * sizeof(T);
-  kp_smem_attr(k_kp_fwd_interior<T>, smem);
+  const size_t smem_int = (size_t)(std::max(max_nI, 1) + kKB - 1) / kKB * kKB * sizeof(T);
+  kp_smem_attr(k_kp_fwd_interior<T>, smem_int);
   kp_smem_attr(k_kp_fwd_boundary<T>, smem);
-  k_kp_fwd_interior<T><<<P, kT, smem, st>>>(lay, Lc, r, yI);
+  k_kp_fwd_interior<T><<<P, kT, smem_int, st>>>(lay, Lc, r, yI);
   const int nblk = std::max(1, (max_nr + 31) / 32);
   k_kp_fwd_boundary<T><<<dim3(nblk, P), kT, smem, st>>>(lay, Lc, r, yI, zb);
 }
 
 template <typename T>
 void kp_backward(int P, const SubLayout* lay, const T* Lc, T* yI, const double* xb, double* x, int init,
-                 int max_nr, cudaStream_t st) {
+                 int max_nr, int max_nI, cudaStream_t st) {
   if (P <= 0) return;
   const size_t smem = (size_t)std::max(max_nr, 1) * sizeof(T);
+  const size_t row = (size_t)(std::max(max_nI, 1) + kKB - 1) / kKB * kKB * sizeof(T);
+  const int parts = 5 * row <= 200 * 1024 ? 4 : 1;
   kp_smem_attr(k_kp_bwd_boundary<T>, smem);
-  kp_smem_attr(k_kp_bwd_interior<T>, smem);
+  kp_smem_attr(k_kp_bwd_interior<T>, (1 + parts) * row);
   const int nblk = std::max(1, (max_nr + 31) / 32);
   k_kp_bwd_boundary<T><<<dim3(nblk, P), kT, smem, st>>>(lay, Lc, xb, yI);
-  k_kp_bwd_interior<T><<<P, kT, smem, st>>>(lay, Lc, yI, xb, x, init);
+  k_kp_bwd_interior<T><<<P, kT, (1 + parts) * row, st>>>(lay, Lc, yI, xb, x, init, parts);
 }
 
 void launch_kp_forward(int P, const SubLayout* lay, const float* Lc, const double* r, float* yI, float* zb, int max_nr,
-                       cudaStream_t st) {
-  kp_forward<float>(P, lay, Lc, r, yI, zb, max_nr, st);
+                       int max_nI, cudaStream_t st) {
+  kp_forward<float>(P, lay, Lc, r, yI, zb, max_nr, max_nI, st);
 }
 
 void launch_kp_backward(int P, const SubLayout* lay, const float* Lc, float* yI, const double* xb, double* x,
-                        int init, int max_nr, cudaStream_t st) {
-  kp_backward<float>(P, lay, Lc, yI, xb, x, init, max_nr, st);
+                        int init, int max_nr, int max_nI, cudaStream_t st) {
+  kp_backward<float>(P, lay, Lc, yI, xb, x, init, max_nr, max_nI, st);
 }
 
 void launch_kp_forward(int P, const SubLayout* lay, const double* Lc, const double* r, double* yI, double* zb,
-                       int max_nr, cudaStream_t st) {
-  kp_forward<double>(P, lay, Lc, r, yI, zb, max_nr, st);
+                       int max_nr, int max_nI, cudaStream_t st) {
+  kp_forward<double>(P, lay, Lc, r, yI, zb, max_nr, max_nI, st);
 }
 
 void launch_kp_backward(int P, const SubLayout* lay, const double* Lc, double* yI, const double* xb, double* x,
-                        int init, int max_nr, cudaStream_t st) {
-  kp_backward<double>(P, lay, Lc, yI, xb, x, init, max_nr, st);
+                        int init, int max_nr, int max_nI, cudaStream_t st) {
+  kp_backward<double>(P, lay, Lc, yI, xb, x, init, max_nr, max_nI, st);
 }
 
 void launch_compact_factor(int P, int max_rows, const SubLayout* lay, const double* A, double* Lc, cudaStream_t st) {

@@ -234,7 +234,7 @@ struct feti_ctx {
   // the last assembly (0 = exact local tangents)
   double shift = 0.0;
   double refine_res = 0.0;
-  int max_nr = 0;
+  int max_nr = 0, max_nI = 0;
   cudaEvent_t elem_ev[2] = {nullptr, nullptr};
   // block form (several right-hand sides)
   int m_cap = 0;  // allocated nrhs capacity of the block buffers
@@ -968,7 +968,10 @@ feti_status build_decomposition(feti_ctx* ctx) {
   };
   env_tables(env0, ctx->env0, ctx->env_off);
   FETI_TRY(upload(ctx, &ctx->d_env0, ctx->env0));
-  for (const auto& L : ctx->lay) ctx->max_nr = std::max(ctx->max_nr, L.nI + L.nbp);
+  for (const auto& L : ctx->lay) {
+    ctx->max_nr = std::max(ctx->max_nr, L.nI + L.nbp);
+    ctx->max_nI = std::max(ctx->max_nI, L.nI);
+  }
   ctx->nloc_total = voff;
   ctx->cd = coff;
   // dense position lookup per subdomain: local DOF -> dense index
@@ -1571,10 +1574,10 @@ void kresid(feti_ctx* ctx, const double* g, const double* x, double* r) {
 // sweeps confined to the interior rows and the boundary block through the
 // explicit FP32 F_i (the autotuned operator kernel of the PCG).
 void kplus_corr(feti_ctx* ctx, const double* r, double* x, bool init) {
-  feti::launch_kp_forward(ctx->P, ctx->d_lay, ctx->d_Lc32, r, ctx->d_kyI, ctx->d_kzb, ctx->max_nr, ctx->stream);
+  feti::launch_kp_forward(ctx->P, ctx->d_lay, ctx->d_Lc32, r, ctx->d_kyI, ctx->d_kzb, ctx->max_nr, ctx->max_nI, ctx->stream);
   gemv_apply(ctx, 0, ctx->d_zero, true, ctx->d_kzb, ctx->d_kxb);
   feti::launch_kp_backward(ctx->P, ctx->d_lay, ctx->d_Lc32, ctx->d_kyI, ctx->d_kxb, x, init ? 1 : 0, ctx->max_nr,
-                           ctx->stream);
+                           ctx->max_nI, ctx->stream);
 }
 
 // x = K^+ g on full local vectors (zero on the fixing DOFs).  FP64
@@ -1591,9 +1594,9 @@ void kplus(feti_ctx* ctx, const double* g, double* x) {
     return;
   }
   if (!f32_factor(ctx)) {
-    feti::launch_kp_forward(ctx->P, ctx->d_lay, ctx->d_Lc, g, ctx->d_kyI64, ctx->d_kzb64, ctx->max_nr, st);
+    feti::launch_kp_forward(ctx->P, ctx->d_lay, ctx->d_Lc, g, ctx->d_kyI64, ctx->d_kzb64, ctx->max_nr, ctx->max_nI, st);
     gemv_apply(ctx, 0, ctx->d_zero, false, ctx->d_kzb64, ctx->d_kxb);
-    feti::launch_kp_backward(ctx->P, ctx->d_lay, ctx->d_Lc, ctx->d_kyI64, ctx->d_kxb, x, 1, ctx->max_nr, st);
+    feti::launch_kp_backward(ctx->P, ctx->d_lay, ctx->d_Lc, ctx->d_kyI64, ctx->d_kxb, x, 1, ctx->max_nr, ctx->max_nI, st);
     return;
   }
   kplus_corr(ctx, g, x, true);
@@ -1706,12 +1709,12 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, double* S64, float* S32,
         rows[phase][t] = std::max(rows[phase][t], m);
       }
     }
-  e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g], A,
-                                ctx->d_cholz, ctx->d_status, st);
+  e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g],
+                                Lc ? 1 : 0, A, ctx->d_cholz, ctx->d_status, st);
   if (e != cudaSuccess) return e;
   if (ctx->opt.precond == FETI_PREC_DIRICHLET)
     feti::launch_extract_tiles(pg, ctx->max_nb, lw, 0, A, S64, S32, S32s, st);
-  e = feti::launch_chol_batched(pg, lw, 1, rows[1].data(), (int)rows[1].size(), nullptr, A, ctx->d_cholz,
+  e = feti::launch_chol_batched(pg, lw, 1, rows[1].data(), (int)rows[1].size(), nullptr, 0, A, ctx->d_cholz,
                                 ctx->d_status, st);
   if (e != cudaSuccess) return e;
   feti::launch_extract_tiles(pg, ctx->max_nb, lw, 1, A, F64, F32, F32s, st);

@@ -303,14 +303,16 @@ namespace feti {
 // nbact boundary rows, the fixing rows), phase 1 the remaining rows plus the
 // augmentation rows of the columns eliminated so far (env0 unused).
 // step_rows[t] (host array, n_steps entries): the largest number of those rows
-// over the subdomains at step t.  Z: scratch, chol_scratch_bytes per subdomain
+// over the subdomains at step t.  winv: store the inverses of the diagonal
+// blocks in place of the blocks (the sweeps over the compact factor multiply
+// by them).  Z: scratch, chol_scratch_bytes per subdomain
 // at SubLayout::zoff.
 constexpr int kCholPanel = 64;
 int64_t chol_scratch_bytes(int n, int elem_bytes);
 cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
-                                const int32_t* env0, double* A, uint8_t* Z, int* status, cudaStream_t st);
+                                const int32_t* env0, int winv, double* A, uint8_t* Z, int* status, cudaStream_t st);
 cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
-                                const int32_t* env0, float* A, uint8_t* Z, int* status, cudaStream_t st);
+                                const int32_t* env0, int winv, float* A, uint8_t* Z, int* status, cudaStream_t st);
 }  // namespace feti
 
 namespace feti {
@@ -337,13 +339,13 @@ void launch_extract_tiles(int P, int max_m, const SubLayout* lay, int which, con
 // pass (forward, FP64 F_i apply, backward: K_rr^-1 by its block form with
 // the Schur complement inverse F_i).
 void launch_kp_forward(int P, const SubLayout* lay, const float* Lc, const double* r, float* yI, float* zb, int max_nr,
-                       cudaStream_t st);
+                       int max_nI, cudaStream_t st);
 void launch_kp_backward(int P, const SubLayout* lay, const float* Lc, float* yI, const double* xb, double* x,
-                        int init, int max_nr, cudaStream_t st);
+                        int init, int max_nr, int max_nI, cudaStream_t st);
 void launch_kp_forward(int P, const SubLayout* lay, const double* Lc, const double* r, double* yI, double* zb,
-                       int max_nr, cudaStream_t st);
+                       int max_nr, int max_nI, cudaStream_t st);
 void launch_kp_backward(int P, const SubLayout* lay, const double* Lc, double* yI, const double* xb, double* x,
-                        int init, int max_nr, cudaStream_t st);
+                        int init, int max_nr, int max_nI, cudaStream_t st);
 // Copies rows [0, nI + nbp) x columns [0, nI) of each eliminated workspace
 // matrix (at lay[s].aoff in A) into the compact interior factor Lc (at
 // lay[s].loff, row stride kp_ld; zero above the diagonal of L_II and in the
