@@ -114,6 +114,8 @@ struct feti_ctx {
   int tuned_m = 0;                     // nrhs the block schedules were tuned for
   bool tuned = false;
   float* d_vloc32 = nullptr;
+  int2* d_chunk_gp = nullptr;  // first boundary position and count of each chunk
+  int4* d_pos_tab = nullptr;
   int32_t *d_chunk_sub = nullptr, *d_chunk_p0 = nullptr, *d_sub_chunk_ptr = nullptr, *d_col_sub = nullptr;
   double* d_gpart = nullptr;
   int32_t *d_gs_ptr = nullptr, *d_gs_pos = nullptr, *d_dir_dof = nullptr;
@@ -1364,6 +1366,14 @@ feti_status build_decomposition(feti_ctx* ctx) {
   }
   FETI_TRY(upload(ctx, &ctx->d_chunk_sub, chunk_sub));
   FETI_TRY(upload(ctx, &ctx->d_chunk_p0, chunk_p0));
+  {
+    std::vector<int2> gp(chunk_sub.size());
+    for (size_t c = 0; c < gp.size(); ++c) {
+      const SubLayout& L = ctx->lay[chunk_sub[c]];
+      gp[c] = make_int2(L.boff + chunk_p0[c], std::min(256, L.nbp + L.k - chunk_p0[c]));
+    }
+    FETI_TRY(upload(ctx, &ctx->d_chunk_gp, gp));
+  }
   FETI_TRY(upload(ctx, &ctx->d_sub_chunk_ptr, sub_chunk_ptr));
   FETI_TRY(upload(ctx, &ctx->d_col_sub, col_sub));
   FETI_TRY(dev_alloc(ctx, &ctx->d_gpart, 6 * (size_t)std::max(ctx->n_chunks, 1)));
@@ -1481,6 +1491,10 @@ feti_status build_decomposition(feti_ctx* ctx) {
   ctx->maps.bt_row = ctx->d_bt_row;
   ctx->maps.bt_sgn = ctx->d_bt_sgn;
   ctx->maps.bpos_sub = ctx->d_bpos_sub;
+  FETI_TRY(dev_alloc(ctx, &ctx->d_pos_tab, (size_t)ctx->nb_total));
+  feti::launch_pos_table((int)ctx->nb_total, ctx->d_bpos_sub, ctx->d_lay, ctx->d_pos_tab, ctx->stream);
+  FETI_CK(cudaGetLastError());
+  ctx->maps.pos_tab = ctx->d_pos_tab;
   FETI_CK(cudaStreamSynchronize(ctx->stream));
   return FETI_OK;
 }
@@ -1860,13 +1874,13 @@ void project(feti_ctx* ctx, const double* v, double* out, const double* a, bool 
   if (!partial) partial = ctx->d_partial;
   if (ctx->cd == 0) {
     // no coarse space: out = v (the expand kernel with c unused)
-    feti::launch_expand(ctx->maps, ctx->d_lay, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
+    feti::launch_expand(ctx->maps, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
     return;
   }
-  feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_sub, ctx->d_chunk_p0, ctx->d_lay, ctx->d_R, ctx->maps, v,
+  feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_gp, ctx->d_R, ctx->maps, v,
                         ctx->d_gpart, done, st);
   coarse_apply_part(ctx, done);
-  feti::launch_expand(ctx->maps, ctx->d_lay, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
+  feti::launch_expand(ctx->maps, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
 }
 
 // Dense local apply of F_i (which 0) or the preconditioner block (which 1)
@@ -2205,13 +2219,13 @@ void pcg_iteration(feti_ctx* ctx, double* lam, bool f32) {
   local_apply(ctx, 0, ctx->d_p, nullptr, done, f32);                              // q = F p, (p, q)
   feti::launch_scatter(ctx->maps, ctx->d_loc, nullptr, ctx->d_q, ctx->d_p, ctx->d_partial_pq, done, st);
   if (ctx->cd > 0) {
-    feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_sub, ctx->d_chunk_p0, ctx->d_lay, ctx->d_R, ctx->maps,
-                          ctx->d_r, ctx->d_gpart, done, st, ctx->d_q, ctx->d_partial_pq, ctx->d_sc,
-                          ctx->d_alpha_hist);
+    feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_gp, ctx->d_R, ctx->maps, ctx->d_r, ctx->d_gpart, done, st,
+                          ctx->d_q, ctx->d_partial_pq, ctx->d_sc, ctx->d_alpha_hist);
     coarse_apply_part(ctx, done);
   }
-  feti::launch_expand_update(ctx->maps, ctx->d_lay, ctx->d_R, ctx->d_r, ctx->d_c, ctx->d_w, ctx->d_partial, lam,
-                             ctx->d_p, ctx->d_q, ctx->d_partial_pq, ctx->d_sc, ctx->d_alpha_hist, st);
+  feti::launch_expand_update(ctx->maps, ctx->d_R, ctx->d_r, ctx->d_c, ctx->d_w, ctx->d_partial, lam,
+                             ctx->d_p, ctx->d_q, ctx->d_partial_pq, ctx->d_sc, ctx->d_alpha_hist, ctx->cd > 0 ? 1 : 0,
+                             st);
   feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, 0, st);
 }
 
@@ -2365,7 +2379,7 @@ feti_status rhs_setup(feti_ctx* ctx) {
   if (ctx->cd > 0) {
     feti::launch_rtx(ctx->P, ctx->d_lay, ctx->d_R, ctx->d_f, -1.0, ctx->d_e, st);
     coarse_apply_g(ctx, ctx->d_e, ctx->d_c, zero);
-    feti::launch_expand(ctx->maps, ctx->d_lay, ctx->d_R, ctx->d_lam, ctx->d_c, ctx->d_lam, nullptr, nullptr, 0,
+    feti::launch_expand(ctx->maps, ctx->d_R, ctx->d_lam, ctx->d_c, ctx->d_lam, nullptr, nullptr, 0,
                         zero, st);
   }
   FETI_CK(cudaGetLastError());

@@ -118,7 +118,11 @@ struct Maps {
   const int32_t* bt_row;    // rows of each boundary position
   const double* bt_sgn;
   const int32_t* bpos_sub;  // [nb_total] owning subdomain of each boundary position
+  const int4* pos_tab;      // [nb_total] kernel dimension, first coarse column and offset of the
+                            // R_i row (low, high word) of each boundary position
 };
+// Fills pos_tab (nb_total entries) from the layouts.
+void launch_pos_table(int nb_total, const int32_t* bpos_sub, const SubLayout* lay, int4* tab, cudaStream_t st);
 
 // y_b = (B_i^T (wv o x))_b: signed gather onto the boundary positions.
 void launch_gather(const Maps& mp, const double* x, const double* wv, double* y, const int* done,
@@ -135,7 +139,7 @@ void launch_gtv(int P, const SubLayout* lay, const double* R, const Maps& mp, co
 void launch_coarse_apply(int cd, const double* Ginv, const double* g, double* c, const int* done,
                          cudaStream_t st);
 // out = v - G c row-wise; optional partial sums of (a, out) (a NULL: (out,out)).
-void launch_expand(const Maps& mp, const SubLayout* lay, const double* R, const double* v, const double* c,
+void launch_expand(const Maps& mp, const double* R, const double* v, const double* c,
                    double* out, const double* a, double* partial, int with_dot, const int* done,
                    cudaStream_t st);
 // G^T G assembled per pair block, deterministic (one CTA per block).
@@ -231,18 +235,18 @@ void launch_vadd(int n, double* a, const double* b, cudaStream_t st);
 
 namespace feti {
 // G^T x over chunks of 256 boundary positions of the subdomains with k > 0:
-// partial[6 c + a] for chunk c.
+// partial[6 c + a] for chunk c; chunk_gp: first boundary position and count.
 // With q != NULL the gathered input is x - alpha q (fused CG update, alpha
 // from the (p, q) partial sums; CTA 0 stores alpha in sc and alpha_hist).
-void launch_gtv_part(int n_chunks, const int32_t* chunk_sub, const int32_t* chunk_p0, const SubLayout* lay,
-                     const double* R, const Maps& mp, const double* x, double* partial, const int* done,
-                     cudaStream_t st, const double* q = nullptr, const double* pq_partial = nullptr,
-                     PcgScalars* sc = nullptr, double* alpha_hist = nullptr);
+void launch_gtv_part(int n_chunks, const int2* chunk_gp, const double* R, const Maps& mp, const double* x,
+                     double* partial, const int* done, cudaStream_t st, const double* q = nullptr,
+                     const double* pq_partial = nullptr, PcgScalars* sc = nullptr, double* alpha_hist = nullptr);
 // Fused CG update + projection expand: r -= alpha q, lam += alpha p in place,
 // out = r - G c, partial sums of ||out||^2.
-void launch_expand_update(const Maps& mp, const SubLayout* lay, const double* R, double* r, const double* c,
-                          double* out, double* partial, double* lam, const double* p, const double* q,
-                          const double* pq_partial, PcgScalars* sc, double* alpha_hist, cudaStream_t st);
+// have_alpha: launch_gtv_part has left this iteration's alpha in sc.
+void launch_expand_update(const Maps& mp, const double* R, double* r, const double* c, double* out, double* partial,
+                          double* lam, const double* p, const double* q, const double* pq_partial, PcgScalars* sc,
+                          double* alpha_hist, int have_alpha, cudaStream_t st);
 // Fused CG step: rho from partial sums, beta, p = y + beta p.
 void launch_axpby_rho(int n, double* p, const double* y, PcgScalars* s, const double* partial, double* beta_hist,
                       cudaStream_t st);

@@ -7,6 +7,7 @@
 // row-major and deterministic (no floating-point atomics anywhere); every
 // subdomain of uneven size is one batch element of a single launch.
 #include "feti_internal.h"
+#include "feti_launch.cuh"
 
 #include <cmath>
 
@@ -664,6 +665,12 @@ __global__ void __launch_bounds__(kThreads) k_gemv_loc(const int32_t* __restrict
                                                        const SubLayout* __restrict__ lay, int which,
                                                        const T* __restrict__ M, const T* __restrict__ vloc,
                                                        double* __restrict__ y, const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  M = fresh(M);
+  vloc = fresh(vloc);
+  y = fresh(y);
+  done = fresh(done);
   if (*done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* v = reinterpret_cast<T*>(smem_raw);
@@ -735,6 +742,11 @@ __global__ void __launch_bounds__(kThreads) k_gemv_loc(const int32_t* __restrict
 // Signed gather onto the boundary positions in FP32 (input of the FP32 apply).
 __global__ void k_gather32(Maps mp, const double* __restrict__ x, const double* __restrict__ wv,
                            float* __restrict__ y, const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  x = fresh(x);
+  y = fresh(y);
+  done = fresh(done);
   if (*done) return;
   for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < mp.nb_total; gp += gridDim.x * blockDim.x) {
     double val = 0.0;
@@ -1081,6 +1093,11 @@ __global__ void __launch_bounds__(SYM_WPC * 32) k_symv2_f32(const int32_t* __res
 // transposed products at column c, in that order.
 __global__ void k_symv_fix(Maps mp, const SubLayout* __restrict__ lay, int which, const float* __restrict__ part,
                            double* __restrict__ y, const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  part = fresh(part);
+  y = fresh(y);
+  done = fresh(done);
   constexpr int PH = kSymPH;
   if (*done) return;
   for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < mp.nb_total; gp += gridDim.x * blockDim.x) {
@@ -1114,6 +1131,11 @@ __global__ void k_vadd(int n, double* __restrict__ a, const double* __restrict__
 
 __global__ void k_gather(Maps mp, const double* __restrict__ x, const double* __restrict__ wv,
                          double* __restrict__ y, const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  x = fresh(x);
+  y = fresh(y);
+  done = fresh(done);
   if (*done) return;
   for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < mp.nb_total; gp += gridDim.x * blockDim.x) {
     double val = 0.0;
@@ -1129,6 +1151,13 @@ __global__ void __launch_bounds__(kThreads) k_scatter(Maps mp, const double* __r
                                                       const double* __restrict__ wv, double* __restrict__ q,
                                                       const double* __restrict__ a, double* __restrict__ partial,
                                                       const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  y = fresh(y);
+  q = fresh(q);
+  a = fresh(a);
+  partial = fresh(partial);
+  done = fresh(done);
   if (*done) return;
   __shared__ double red[32];
   double dot = 0.0;
@@ -1178,20 +1207,38 @@ __device__ double reduce_partials(const double* partial, double* red) {
   return block_sum(t, red);
 }
 
+__device__ __forceinline__ int64_t pos_roff(const int4& t) {
+  return (int64_t)(((uint64_t)(uint32_t)t.w << 32) | (uint32_t)t.z);
+}
+__global__ void k_pos_table(int nb_total, const int32_t* __restrict__ bpos_sub, const SubLayout* __restrict__ lay,
+                            int4* __restrict__ tab) {
+  for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < nb_total; gp += gridDim.x * blockDim.x) {
+    const SubLayout& L = lay[bpos_sub[gp]];
+    const uint64_t o = (uint64_t)(L.roff + (int64_t)(L.nI + gp - L.boff) * L.k);
+    tab[gp] = make_int4(L.k, L.coff, (int)(uint32_t)o, (int)(uint32_t)(o >> 32));
+  }
+}
+
 // G^T x split over chunks of 256 boundary positions (one CTA per chunk,
 // several per subdomain): partial[c*6 + a] = sum over the chunk of
 // R_b[p][a] (B^T x)[p].
 // With q != NULL the input is the updated residual x - alpha q, alpha =
 // rho / (p, q) evaluated by every CTA from the partial sums of (p, q) (the
 // fused CG step); CTA 0 records alpha and flags a breakdown.
-__global__ void __launch_bounds__(kThreads) k_gtv_part(const int32_t* __restrict__ chunk_sub,
-                                                       const int32_t* __restrict__ chunk_p0, int n_chunks,
-                                                       const SubLayout* __restrict__ lay,
+__global__ void __launch_bounds__(kThreads) k_gtv_part(const int2* __restrict__ chunk_gp, int n_chunks,
                                                        const double* __restrict__ R, Maps mp,
                                                        const double* __restrict__ x, double* __restrict__ partial,
                                                        const int* __restrict__ done, const double* __restrict__ q,
                                                        const double* __restrict__ pq_partial, PcgScalars* sc,
                                                        double* __restrict__ alpha_hist) {
+  dep_wait();
+  dep_go();
+  x = fresh(x);
+  partial = fresh(partial);
+  done = fresh(done);
+  q = fresh(q);
+  pq_partial = fresh(pq_partial);
+  sc = fresh(sc);
   if (*done) return;
   __shared__ double red[32];
   double alpha = 0.0;
@@ -1215,19 +1262,20 @@ __global__ void __launch_bounds__(kThreads) k_gtv_part(const int32_t* __restrict
   const int c = blockIdx.x;
   if (c >= n_chunks) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const SubLayout L = lay[chunk_sub[c]];
-  const int nb = L.nbp + L.k;
-  const int p = chunk_p0[c] + threadIdx.x;
+  const int2 ch = __ldg(chunk_gp + c);
   double v8[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (p < nb) {
-    const int gp = L.boff + p;
+  if ((int)threadIdx.x < ch.y) {
+    const int gp = ch.x + threadIdx.x;
+    const int4 tab = __ldg(mp.pos_tab + gp);
     double val = 0.0;
     for (int e = mp.bt_ptr[gp]; e < mp.bt_ptr[gp + 1]; ++e) {
       const int row = mp.bt_row[e];
       val += mp.bt_sgn[e] * (q ? x[row] - alpha * q[row] : x[row]);
     }
-    const double* Rr = R + L.roff + (size_t)(L.nI + p) * L.k;
-    for (int a = 0; a < L.k; ++a) v8[a] = Rr[a] * val;
+    const double* Rr = R + pos_roff(tab);
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+      if (a < tab.x) v8[a] = Rr[a] * val;
   }
   // step 16: keep half the values, add the partner's copy of that half
   double v4[4], v2[2], v1;
@@ -1265,7 +1313,7 @@ __global__ void __launch_bounds__(kThreads) k_gtv_part(const int32_t* __restrict
     wsum[wid][a] = v1;
   }
   __syncthreads();
-  if (threadIdx.x < L.k) {
+  if (threadIdx.x < 6) {  // zero beyond the kernel dimension
     double t = 0.0;
     for (int w = 0; w < kThreads / 32; ++w) t += wsum[w][threadIdx.x];
     partial[6 * c + threadIdx.x] = t;
@@ -1278,6 +1326,12 @@ __global__ void k_coarse_apply_part(int cd, const double* __restrict__ Ginv, con
                                     const int32_t* __restrict__ sub_chunk_ptr, const int32_t* __restrict__ col_sub,
                                     const SubLayout* __restrict__ lay, double* __restrict__ c,
                                     const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  Ginv = fresh(Ginv);
+  partial = fresh(partial);
+  c = fresh(c);
+  done = fresh(done);
   if (*done) return;
   extern __shared__ double gsh[];
   for (int j = threadIdx.x; j < cd; j += blockDim.x) {
@@ -1323,17 +1377,33 @@ struct ExpandUpdate {
   const double* pq_partial;
   PcgScalars* sc;
   double* alpha_hist;
+  int have_alpha;  // alpha of this iteration is in sc already
 };
 
-__global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const SubLayout* __restrict__ lay,
-                                                     const double* __restrict__ R, const double* __restrict__ v,
+__global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const double* __restrict__ R, const double* __restrict__ v,
                                                      const double* __restrict__ c, double* __restrict__ out,
                                                      const double* __restrict__ a, double* __restrict__ partial,
                                                      int with_dot, const int* __restrict__ done, ExpandUpdate upd) {
+  dep_wait();
+  dep_go();
+  v = fresh(v);
+  c = fresh(c);
+  out = fresh(out);
+  a = fresh(a);
+  partial = fresh(partial);
+  done = fresh(done);
+  upd.r = fresh(upd.r);
+  upd.lam = fresh(upd.lam);
+  upd.p = fresh(upd.p);
+  upd.q = fresh(upd.q);
+  upd.pq_partial = fresh(upd.pq_partial);
+  upd.sc = fresh(upd.sc);
   if (*done) return;
   __shared__ double red[32];
   double alpha = 0.0;
-  if (upd.r) {
+  if (upd.r && upd.have_alpha) {
+    alpha = upd.sc->alpha;
+  } else if (upd.r) {
     const double pq = reduce_partials(upd.pq_partial, red);
     alpha = upd.sc->rho / pq;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1360,11 +1430,16 @@ __global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const SubLayout* _
     for (int e = 0; e < 2; ++e) {
       const int gp = mp.row_pos[2 * r + e];
       if (gp >= 0) {
-        const SubLayout L = lay[mp.bpos_sub[gp]];
-        if (L.k) {
-          const double* Rr = R + L.roff + (size_t)(L.nI + gp - L.boff) * L.k;
+        const int4 tab = __ldg(mp.pos_tab + gp);
+        if (tab.x) {
+          const double* Rr = R + pos_roff(tab);
           double t = 0.0;
-          for (int k = 0; k < L.k; ++k) t += Rr[k] * c[L.coff + k];
+          if (tab.x == 6) {  // a floating subdomain: all twelve loads at once
+#pragma unroll
+            for (int k = 0; k < 6; ++k) t += Rr[k] * c[tab.y + k];
+          } else {
+            for (int k = 0; k < tab.x; ++k) t += Rr[k] * c[tab.y + k];
+          }
           val -= mp.row_sgn[2 * r + e] * t;
         }
       }
@@ -1409,6 +1484,10 @@ __global__ void k_gtg(const int32_t* __restrict__ blk_i, const int32_t* __restri
 // ---------------------------------------------------------------------------
 
 __global__ void k_ctl_conv(PcgScalars* s, const double* __restrict__ partial, int first) {
+  dep_wait();
+  dep_go();
+  s = fresh(s);
+  partial = fresh(partial);
   if (s->done) return;
   __shared__ double red[32];
   const double wn = sqrt(reduce_partials(partial, red));
@@ -1440,6 +1519,12 @@ __global__ void k_ctl_conv(PcgScalars* s, const double* __restrict__ partial, in
 __global__ void __launch_bounds__(kThreads) k_axpby_rho(int n, double* __restrict__ p, const double* __restrict__ y,
                                                         PcgScalars* s, const double* __restrict__ partial,
                                                         double* __restrict__ beta_hist) {
+  dep_wait();
+  dep_go();
+  p = fresh(p);
+  y = fresh(y);
+  s = fresh(s);
+  partial = fresh(partial);
   if (s->done) return;
   __shared__ double red[32];
   const double rho = reduce_partials(partial, red);
@@ -1617,12 +1702,12 @@ void launch_kplus(int P, const SubLayout* lay, const double* A, const double* g,
 
 void launch_gather(const Maps& mp, const double* x, const double* wv, double* y, const int* done,
                    cudaStream_t st) {
-  k_gather<<<grid_for(mp.nb_total), kThreads, 0, st>>>(mp, x, wv, y, done);
+  (void)launch_dep(k_gather, dim3(grid_for(mp.nb_total)), dim3(kThreads), 0, st, mp, x, wv, y, done);
 }
 
 void launch_scatter(const Maps& mp, const double* y, const double* wv, double* q, const double* a,
                     double* partial, const int* done, cudaStream_t st) {
-  k_scatter<<<kPartials, kThreads, 0, st>>>(mp, y, wv, q, a, partial, done);
+  (void)launch_dep(k_scatter, dim3(kPartials), dim3(kThreads), 0, st, mp, y, wv, q, a, partial, done);
 }
 
 void launch_gtv(int P, const SubLayout* lay, const double* R, const Maps& mp, const double* x, double* g,
@@ -1637,10 +1722,10 @@ void launch_coarse_apply(int cd, const double* Ginv, const double* g, double* c,
   k_coarse_apply<<<(warps * 32 + kThreads - 1) / kThreads, kThreads, 0, st>>>(cd, Ginv, g, c, done);
 }
 
-void launch_expand(const Maps& mp, const SubLayout* lay, const double* R, const double* v, const double* c,
+void launch_expand(const Maps& mp, const double* R, const double* v, const double* c,
                    double* out, const double* a, double* partial, int with_dot, const int* done,
                    cudaStream_t st) {
-  k_expand<<<kPartials, kThreads, 0, st>>>(mp, lay, R, v, c, out, a, partial, with_dot, done, ExpandUpdate{});
+  (void)launch_dep(k_expand, dim3(kPartials), dim3(kThreads), 0, st, mp, R, v, c, out, a, partial, with_dot, done, ExpandUpdate{});
 }
 
 void launch_gtg(int n_blocks, const int32_t* blk_i, const int32_t* blk_j, const int32_t* blk_ptr,
@@ -1651,7 +1736,7 @@ void launch_gtg(int n_blocks, const int32_t* blk_i, const int32_t* blk_j, const 
 }
 
 void launch_ctl_conv(PcgScalars* s, const double* partial, int first, cudaStream_t st) {
-  k_ctl_conv<<<1, kThreads, 0, st>>>(s, partial, first);
+  (void)launch_dep(k_ctl_conv, dim3(1), dim3(kThreads), 0, st, s, partial, first);
 }
 void launch_vsub(int n, const double* a, const double* b, double* out, cudaStream_t st) {
   k_vsub<<<grid_for(n), kThreads, 0, st>>>(n, a, b, out);
@@ -1685,7 +1770,7 @@ static void launch_gemv_t(int n_blocks, const int32_t* blk_sub, const int32_t* b
                           cudaStream_t st) {
   const size_t smem = (size_t)((max_m + 3) & ~3) * sizeof(T);
   if (smem > 48 * 1024) cudaFuncSetAttribute(k_gemv_loc<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_gemv_loc<T, R><<<n_blocks, kThreads, smem, st>>>(blk_sub, blk_row0, rpc, lay, which, M, vloc, y, done);
+  (void)launch_dep(k_gemv_loc<T, R>, dim3(n_blocks), dim3(kThreads), smem, st, blk_sub, blk_row0, rpc, lay, which, M, vloc, y, done);
 }
 
 void launch_gemv_loc(const GemvCfg& cfg, const SubLayout* lay, int which, const void* M, int f32, const void* vloc,
@@ -1714,15 +1799,18 @@ void launch_symv_f32(int G, int n_warps, const int32_t* wsub, const int32_t* wpa
                      cudaStream_t st) {
   const int blocks = (n_warps + kThreads / 32 - 1) / (kThreads / 32);
   // G: rows per load group (8, 16, 32); + 100 * PF: L2 prefetch PF tiles ahead (1, 2)
+  auto go = [&](auto kern) {
+    kern<<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done);
+  };
   switch (G) {
-    case 8: k_symv_f32<8, 0><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
-    case 16: k_symv_f32<16, 0><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
-    case 108: k_symv_f32<8, 1><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
-    case 132: k_symv_f32<32, 1><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
-    case 232: k_symv_f32<32, 2><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
-    default: k_symv_f32<32, 0><<<blocks, kThreads, 0, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done); break;
+    case 8: go(k_symv_f32<8, 0>); break;
+    case 16: go(k_symv_f32<16, 0>); break;
+    case 108: go(k_symv_f32<8, 1>); break;
+    case 132: go(k_symv_f32<32, 1>); break;
+    case 232: go(k_symv_f32<32, 2>); break;
+    default: go(k_symv_f32<32, 0>); break;
   }
-  k_symv_fix<<<grid_for(mp.nb_total), kThreads, 0, st>>>(mp, lay, which, part, y, done);
+  (void)launch_dep(k_symv_fix, dim3(grid_for(mp.nb_total)), dim3(kThreads), 0, st, mp, lay, which, part, y, done);
 }
 
 void launch_symv3_f32(int G, int P, const int32_t* order, int max_m, const SubLayout* lay, int which,
@@ -1753,36 +1841,40 @@ void launch_symv2_f32(int n_warps, const int32_t* wsub, const int32_t* wpanel, c
   const int blocks = (n_warps + SYM_WPC - 1) / SYM_WPC;
   k_symv2_f32<<<blocks, SYM_WPC * 32, smem, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done, err,
                                                   spin_cycles);
-  k_symv_fix<<<grid_for(mp.nb_total), kThreads, 0, st>>>(mp, lay, which, part, y, done);
+  (void)launch_dep(k_symv_fix, dim3(grid_for(mp.nb_total)), dim3(kThreads), 0, st, mp, lay, which, part, y, done);
 }
 
 void launch_gather32(const Maps& mp, const double* x, const double* wv, float* y, const int* done, cudaStream_t st) {
-  k_gather32<<<grid_for(mp.nb_total), kThreads, 0, st>>>(mp, x, wv, y, done);
+  (void)launch_dep(k_gather32, dim3(grid_for(mp.nb_total)), dim3(kThreads), 0, st, mp, x, wv, y, done);
 }
 
 void launch_vadd(int n, double* a, const double* b, cudaStream_t st) {
   k_vadd<<<grid_for(n), kThreads, 0, st>>>(n, a, b);
 }
 
-void launch_gtv_part(int n_chunks, const int32_t* chunk_sub, const int32_t* chunk_p0, const SubLayout* lay,
-                     const double* R, const Maps& mp, const double* x, double* partial, const int* done,
-                     cudaStream_t st, const double* q, const double* pq_partial, PcgScalars* sc,
-                     double* alpha_hist) {
+void launch_gtv_part(int n_chunks, const int2* chunk_gp, const double* R, const Maps& mp, const double* x,
+                     double* partial, const int* done, cudaStream_t st, const double* q, const double* pq_partial,
+                     PcgScalars* sc, double* alpha_hist) {
   if (n_chunks <= 0) return;
-  k_gtv_part<<<n_chunks, kThreads, 0, st>>>(chunk_sub, chunk_p0, n_chunks, lay, R, mp, x, partial, done, q,
-                                            pq_partial, sc, alpha_hist);
+  (void)launch_dep(k_gtv_part, dim3(n_chunks), dim3(kThreads), 0, st, chunk_gp, n_chunks, R, mp, x, partial, done, q,
+                   pq_partial, sc, alpha_hist);
 }
 
-void launch_expand_update(const Maps& mp, const SubLayout* lay, const double* R, double* r, const double* c,
-                          double* out, double* partial, double* lam, const double* p, const double* q,
-                          const double* pq_partial, PcgScalars* sc, double* alpha_hist, cudaStream_t st) {
-  ExpandUpdate u{r, lam, p, q, pq_partial, sc, alpha_hist};
-  k_expand<<<kPartials, kThreads, 0, st>>>(mp, lay, R, r, c, out, nullptr, partial, 1, &sc->done, u);
+void launch_pos_table(int nb_total, const int32_t* bpos_sub, const SubLayout* lay, int4* tab, cudaStream_t st) {
+  if (nb_total > 0) k_pos_table<<<grid_for(nb_total), kThreads, 0, st>>>(nb_total, bpos_sub, lay, tab);
+}
+
+void launch_expand_update(const Maps& mp, const double* R, double* r, const double* c, double* out, double* partial,
+                          double* lam, const double* p, const double* q, const double* pq_partial, PcgScalars* sc,
+                          double* alpha_hist, int have_alpha, cudaStream_t st) {
+  ExpandUpdate u{r, lam, p, q, pq_partial, sc, alpha_hist, have_alpha};
+  (void)launch_dep(k_expand, dim3(kPartials), dim3(kThreads), 0, st, mp, R, r, c, out, nullptr, partial, 1, &sc->done,
+                   u);
 }
 
 void launch_axpby_rho(int n, double* p, const double* y, PcgScalars* s, const double* partial, double* beta_hist,
                       cudaStream_t st) {
-  k_axpby_rho<<<grid_for(n), kThreads, 0, st>>>(n, p, y, s, partial, beta_hist);
+  (void)launch_dep(k_axpby_rho, dim3(grid_for(n)), dim3(kThreads), 0, st, n, p, y, s, partial, beta_hist);
 }
 
 void launch_coarse_apply_part(int cd, const double* Ginv, const double* partial, const int32_t* sub_chunk_ptr,
@@ -1793,7 +1885,7 @@ void launch_coarse_apply_part(int cd, const double* Ginv, const double* partial,
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_coarse_apply_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int warps = cd < 2432 ? cd : 2432;
-  k_coarse_apply_part<<<(warps * 32 + kThreads - 1) / kThreads, kThreads, smem, st>>>(cd, Ginv, partial,
+  (void)launch_dep(k_coarse_apply_part, dim3((warps * 32 + kThreads - 1) / kThreads), dim3(kThreads), smem, st, cd, Ginv, partial,
                                                                                         sub_chunk_ptr, col_sub, lay,
                                                                                         c, done);
 }
@@ -2080,6 +2172,12 @@ __global__ void __launch_bounds__(kThreads) k_spmv_lump(int n_rows, const int32_
                                                         const double* __restrict__ val,
                                                         const double* __restrict__ v, double* __restrict__ y,
                                                         const int* __restrict__ done) {
+  dep_wait();
+  dep_go();
+  val = fresh(val);
+  v = fresh(v);
+  y = fresh(y);
+  done = fresh(done);
   if (*done) return;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2106,7 +2204,7 @@ void launch_lump_fill(long nnz, const int64_t* src, const float* A, double* val,
 void launch_spmv_lump(int n_rows, const int32_t* ptr, const int32_t* col, const double* val, const double* v,
                       double* y, const int* done, cudaStream_t st) {
   const int warps = n_rows < 65536 ? n_rows : 65536;
-  k_spmv_lump<<<(warps * 32 + kThreads - 1) / kThreads, kThreads, 0, st>>>(n_rows, ptr, col, val, v, y, done);
+  (void)launch_dep(k_spmv_lump, dim3((warps * 32 + kThreads - 1) / kThreads), dim3(kThreads), 0, st, n_rows, ptr, col, val, v, y, done);
 }
 
 namespace {
