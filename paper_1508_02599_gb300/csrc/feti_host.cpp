@@ -1531,11 +1531,14 @@ feti_status check_wait_flag(feti_ctx* ctx, int* d_flag, const char* where) {
 // Element matrices at dU (device or NULL): the two-fibre tangent and force,
 // Hooke P1 (linear, and P2-P0 on P1 where the element mean of div u is div u),
 // or Hooke P2 / P2-P0 on 10-node tetrahedra.
-void launch_elements(feti_ctx* ctx, const double* dU) {
+// Ke_full (two-fibre only): 12 x 12 matrices there and forces in fe instead of
+// the packed ones in d_Ke and d_fe.
+void launch_elements(feti_ctx* ctx, const double* dU, double* Ke_full = nullptr, double* fe = nullptr) {
   cudaStream_t st = ctx->stream;
   if (ctx->mat.kind == FETI_HGO_TWO_FIBRE)
     feti::launch_elem_hgo(ctx->E, ctx->d_coords, ctx->d_tets, dU, ctx->d_fibres, ctx->mat.c, ctx->mat.k1,
-                          ctx->mat.k2, ctx->mat.kappa, ctx->d_Ke, ctx->d_fe, ctx->d_status, st);
+                          ctx->mat.k2, ctx->mat.kappa, Ke_full ? Ke_full : ctx->d_Ke, Ke_full ? fe : ctx->d_fe,
+                          Ke_full != nullptr, ctx->d_status, st);
   else if (ctx->npe == 10)
     feti::launch_elem_linear_p2(ctx->E, ctx->d_coords, ctx->d_tets, ctx->mat.E, ctx->mat.nu,
                                 ctx->mat.kind == FETI_LINEAR_ISO_P0 ? 1 : 0, ctx->d_Ke, ctx->d_status, st);
@@ -3364,13 +3367,18 @@ feti_status feti_elements(feti_ctx* ctx, const double* U, int32_t u_on_device, d
     FETI_CK(cudaMemcpyAsync(ctx->d_U, U, n3 * sizeof(double), u_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
     dU = ctx->d_U;
   }
+  // Two-fibre matrices for a device array are written in place: 1.16 GB once
+  // (663,552 elements) instead of packed, expanded and the forces copied.  Its
+  // rows are stored 32 bytes at a time; an array that is not aligned to that
+  // takes the packed matrices and the expansion, as do the linear materials.
+  const bool direct = hgo && out_on_device && reinterpret_cast<uintptr_t>(Ke_out) % 32 == 0;
   FETI_CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
   if (!ctx->elem_ev[0]) {
     FETI_CK(cudaEventCreate(&ctx->elem_ev[0]));
     FETI_CK(cudaEventCreate(&ctx->elem_ev[1]));
   }
   FETI_CK(cudaEventRecord(ctx->elem_ev[0], st));
-  launch_elements(ctx, dU);
+  launch_elements(ctx, dU, direct ? Ke_out : nullptr, fe_out);
   FETI_CK(cudaGetLastError());
   FETI_CK(cudaEventRecord(ctx->elem_ev[1], st));
   FETI_TRY(check_status(ctx, "element matrices"));
@@ -3378,13 +3386,16 @@ feti_status feti_elements(feti_ctx* ctx, const double* U, int32_t u_on_device, d
     float ms = 0.f;
     FETI_CK(cudaEventElapsedTime(&ms, ctx->elem_ev[0], ctx->elem_ev[1]));
     ctx->elem_ms = ms;
-    // connectivity, fibres (hyperelastic), packed symmetric tangent and force
-    // per element; coordinates (+ displacement) per node
+    // connectivity, fibres (hyperelastic), symmetric tangent (packed, or full
+    // where it went straight to the caller's array) and force per element;
+    // coordinates (+ displacement) per node
     const double nd = ctx->nde;
-    const double per_elem = 4.0 * ctx->npe + nd * (nd + 1) / 2 * 8.0 + (hgo ? 48.0 + 12.0 * 8.0 : 0.0);
+    const double per_elem =
+        4.0 * ctx->npe + nd * (direct ? nd : (nd + 1) / 2) * 8.0 + (hgo ? 48.0 + 12.0 * 8.0 : 0.0);
     const double per_node = hgo ? 48.0 : 24.0;
     ctx->elem_bytes = per_elem * (double)ctx->E + per_node * (double)ctx->N;
   }
+  if (direct) return FETI_OK;
   const cudaMemcpyKind kind = out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   // full nde x nde copies of the packed (upper-triangle) element matrices
   const size_t full = (size_t)ctx->nde * ctx->nde * ctx->E;

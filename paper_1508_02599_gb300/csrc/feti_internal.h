@@ -70,9 +70,11 @@ __host__ __device__ inline int ke_idx(int nde, int i, int j) {
 void launch_ke_unpack(int n_el, int nde, const double* Kp, double* K, cudaStream_t st);
 void launch_elem_linear(int n_tets, const double* coords, const int32_t* tets, double E, double nu,
                         double* Ke, int* status, cudaStream_t st);
+// full: Ke takes 12 x 12 row-major matrices (32-byte aligned) instead of packed
+// ones (16-byte aligned).
 void launch_elem_hgo(int n_tets, const double* coords, const int32_t* tets, const double* U,
                      const double* fibres, double c, double k1, double k2, double kappa,
-                     double* Ke, double* fe, int* status, cudaStream_t st);
+                     double* Ke, double* fe, bool full, int* status, cudaStream_t st);
 
 // P2 (10-node) linear element matrices [n_tets * 900] (tets: [n_tets * 10]);
 // p0: volumetric part condensed to a piecewise-constant pressure (P2-P0).

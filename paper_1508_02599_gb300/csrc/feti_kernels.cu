@@ -10,6 +10,7 @@
 #include "feti_launch.cuh"
 
 #include <cmath>
+#include <type_traits>
 
 namespace feti {
 
@@ -57,7 +58,7 @@ __device__ __forceinline__ bool p1_gradients(const double x[4][3], double g[4][3
   const double c01 = Jm[1][2] * Jm[2][0] - Jm[1][0] * Jm[2][2];
   const double c02 = Jm[1][0] * Jm[2][1] - Jm[1][1] * Jm[2][0];
   const double det = Jm[0][0] * c00 + Jm[0][1] * c01 + Jm[0][2] * c02;
-  V = det / 6.0;
+  V = det * (1.0 / 6.0);
   if (!(det > 0.0)) return false;
   const double id = 1.0 / det;
   double Ji[3][3];  // inverse of Jm
@@ -191,20 +192,56 @@ __global__ void k_elem_linear_p2(int n_tets, const double* __restrict__ coords, 
 //   c_Q = -2 A_v + (2c/3) J23 I1 + sum_f (4/3) psi'_f J23 I4_f
 //   (dC^-1/dC = -Q, dJ/dC = J/2 C^-1, dJ23/dC = -J23/3 C^-1, dI1/dC = I, dI4/dC = a a).
 //
-// Spatial evaluation.  The tangent block K[(a,i),(b,j)] = V (delta_ij g_a.S g_b
+// Spatial evaluation.  K[(a,i),(b,j)] = V (delta_ij g_a.S g_b
 // + sum F_iI g_aJ CC_IJKL F_jK g_bL) is the same number when every tensor is
 // pushed forward by F: with the current gradients h_a = F^-T g_a, C^-1 -> 1,
-// I -> b = F F^T, a a -> A A (A = F a), Q -> the symmetric identity, S -> the
-// Kirchhoff stress tau = F S F^T, and the tangent becomes
-//   K[(a,i),(b,j)] = V [ c_11 h_ai h_bj + (c_Q/2)(delta_ij h_a.h_b + h_aj h_bi)
-//       + c_IC ((b h_a)_i h_bj + h_ai (b h_b)_j)
-//       + sum_f ( 4 psi''_f J23^2 (beta_f h_a)_i (beta_f h_b)_j
-//                 - (2/3) psi'_f J23 (h_ai w_fbj + w_fai h_bj) )
-//       + delta_ij h_a.tau h_b ],
-//   beta_f = A A - I4/3 1,  w_fa = beta_f h_a + (A.h_a) A,
-// and the internal force f_a = V tau h_a.  Every term is a product of
-// per-node 3-vectors, about a fifth of the FP64 operations of contracting the
-// material tensor entry by entry; all arrays stay in registers.
+// I -> F F^T, a a -> A A (A = F a), Q -> the symmetric identity.  Two vectors
+// per node carry what is left: F F^T h_a = F g_a and A.h_a = a.g_a =: s_fa, so
+// with m_f = 2 psi'_f J23, w = (c J23 I1 + sum_f m_f I4_f) / 3
+//   y_a  = V (c J23 F g_a + sum_f m_f s_fa A_f),   T = V (A_v - w)
+//   p_a  = -(2/3) y_a + V (kappa (2J-1) J / 2 + w/3) h_a
+//   r_fa = 2 J23 sqrt(V psi''_f) (s_fa A_f - I4_f/3 h_a)
+//   K[a,b] = p_a h_b^T + h_a p_b^T - T h_b h_a^T + sum_f r_fa r_fb^T + (h_a.y_b) 1
+//   f_a    = y_a + T h_a
+// (c_Q V/2 = -T, so the stress's own multiple of 1 leaves the diagonal term).
+// The gradients sum to zero over the nodes, hence so do K's block rows and f:
+// only nodes 1..3 are contracted, node 0's blocks are minus the sums.
+//
+// Bound by the FP64 pipe (two lanes a clock and SM): about 740 operations an
+// element against 1210 with all four nodes and the matrices F F^T and tau
+// formed.  The full matrices are written by this kernel as well, a row of 12
+// as three 32-byte stores (whole sectors), instead of being expanded from the
+// packed ones by a second pass.
+struct KeFull {  // row-major 12 x 12, 32-byte aligned
+  static constexpr int kStride = 144;
+  double* K;
+  template <int r>
+  __device__ __forceinline__ void row(const double* v) const {
+#pragma unroll
+    for (int q = 0; q < 12; q += 4)
+      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(K + 12 * r + q), "d"(v[q]), "d"(v[q + 1]),
+                   "d"(v[q + 2]), "d"(v[q + 3])
+                   : "memory");
+  }
+};
+struct KePacked {  // upper triangle, 16-byte aligned
+  static constexpr int kStride = ke_packed(12);
+  double* K;
+  template <int r>
+  __device__ __forceinline__ void row(const double* v) const {
+    constexpr int o = r * 12 - r * (r - 1) / 2;  // entry (r, r)
+    if (o & 1) K[o] = v[r];
+#pragma unroll
+    for (int q = r + (o & 1); q < 12; q += 2) {
+      if (q + 1 < 12)
+        *reinterpret_cast<double2*>(K + o + q - r) = make_double2(v[q], v[q + 1]);
+      else
+        K[o + q - r] = v[q];
+    }
+  }
+};
+
+template <class Out>
 __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __restrict__ coords,
                                                  const int32_t* __restrict__ tets, const double* __restrict__ U,
                                                  const double* __restrict__ fibres, double cmat, double k1,
@@ -233,7 +270,7 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
     for (int j = 0; j < 3; ++j) {
       double s = (i == j) ? 1.0 : 0.0;
 #pragma unroll
-      for (int a = 0; a < 4; ++a) s += u[a][i] * g[a][j];
+      for (int a = 1; a < 4; ++a) s += (u[a][i] - u[0][i]) * g[a][j];
       F[i][j] = s;
     }
   // cofactor matrix: cof(F) = J F^-T
@@ -253,113 +290,141 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
     return;
   }
   const double iJ = 1.0 / J;
-  double h[4][3];  // h_a = F^-T g_a
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int m = 0; m < 3; ++m) h[a][m] = (cf[m][0] * g[a][0] + cf[m][1] * g[a][1] + cf[m][2] * g[a][2]) * iJ;
-  double bm[3][3];  // b = F F^T
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i; j < 3; ++j) {
-      bm[i][j] = F[i][0] * F[j][0] + F[i][1] * F[j][1] + F[i][2] * F[j][2];
-      bm[j][i] = bm[i][j];
-    }
-  const double I1 = bm[0][0] + bm[1][1] + bm[2][2];
   const double J23 = rcbrt(J * J);
-  const double Av = kappa * (J - 1.0) * J;
-  // Kirchhoff stress: tau = t0 1 + c J23 b + sum_f 2 psi'_f J23 A_f A_f
-  double t0 = Av - cmat * J23 * I1 / 3.0;
-  double tau[3][3];
+  const double cJ = cmat * J23;
+  double I1 = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) tau[i][j] = cmat * J23 * bm[i][j];
-  double Af[2][3], I4[2], dpsi[2], d2psi[2];
-  double cQ = -2.0 * Av + 2.0 * cmat * J23 * I1 / 3.0;
+    for (int j = 0; j < 3; ++j) I1 += F[i][j] * F[i][j];
+  // nodes 1..3: h_a = F^-T g_a, y_a
+  double h[3][3], y[3][3], r[2][3][3];
+  const double VcJ = V * cJ;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      h[a][i] = (cf[i][0] * g[a + 1][0] + cf[i][1] * g[a + 1][1] + cf[i][2] * g[a + 1][2]) * iJ;
+      y[a][i] = VcJ * (F[i][0] * g[a + 1][0] + F[i][1] * g[a + 1][1] + F[i][2] * g[a + 1][2]);
+    }
+  double w = cJ * I1;
 #pragma unroll
   for (int f = 0; f < 2; ++f) {
-    double a0[3];
+    double a0[3], A[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) a0[i] = fibres[6 * e + 3 * f + i];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) Af[f][i] = F[i][0] * a0[0] + F[i][1] * a0[1] + F[i][2] * a0[2];
-    I4[f] = Af[f][0] * Af[f][0] + Af[f][1] * Af[f][1] + Af[f][2] * Af[f][2];
-    const double dlt = J23 * I4[f] - 1.0;
+    for (int i = 0; i < 3; ++i) A[i] = F[i][0] * a0[0] + F[i][1] * a0[1] + F[i][2] * a0[2];
+    const double I4 = A[0] * A[0] + A[1] * A[1] + A[2] * A[2];
+    const double dlt = J23 * I4 - 1.0;
+    double dpsi = 0.0, d2psi = 0.0;  // dPsi/dI4bar, d2Psi/dI4bar2
     if (dlt > 1e-12) {
-      const double ex = exp(k2 * dlt * dlt);
-      dpsi[f] = k1 * dlt * ex;                            // dPsi/dI4bar
-      d2psi[f] = k1 * ex * (1.0 + 2.0 * k2 * dlt * dlt);  // d2Psi/dI4bar2
-    } else {
-      dpsi[f] = d2psi[f] = 0.0;
+      const double kd = k2 * dlt * dlt;
+      const double ex = k1 * exp(kd);
+      dpsi = dlt * ex;
+      d2psi = ex * (1.0 + 2.0 * kd);
     }
-    const double m2 = 2.0 * dpsi[f] * J23;
-    t0 -= m2 * I4[f] / 3.0;
+    const double m = 2.0 * dpsi * J23;
+    w += m * I4;
+    const double Vm = V * m;
+    const double cr = 2.0 * J23 * sqrt(V * d2psi);
+    const double ch = cr * I4 * (1.0 / 3.0);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) tau[i][j] += m2 * Af[f][i] * Af[f][j];
-    cQ += 2.0 * m2 * I4[f] / 3.0;
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) tau[i][i] += t0;
-  const double c11 = kappa * (2.0 * J - 1.0) * J + 2.0 * cmat * J23 * I1 / 9.0;
-  const double cIC = -2.0 * cmat * J23 / 3.0;
-  // per-node vectors, scaled by V: P_a = V (c_IC b h_a - (2/3) sum_f psi'_f J23 w_fa),
-  // Pv_a = P_a + V c_11 h_a, r_fa = sqrt(4 V psi''_f) J23 beta_f h_a; tau h_a
-  double P[4][3], Pv[4][3], r[2][4][3], th[4][3];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      th[a][i] = tau[i][0] * h[a][0] + tau[i][1] * h[a][1] + tau[i][2] * h[a][2];
-      P[a][i] = cIC * (bm[i][0] * h[a][0] + bm[i][1] * h[a][1] + bm[i][2] * h[a][2]);
-    }
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const double sa = Af[f][0] * h[a][0] + Af[f][1] * h[a][1] + Af[f][2] * h[a][2];
-      const double cw = -(2.0 / 3.0) * dpsi[f] * J23;
-      const double cr = 2.0 * J23 * sqrt(V * d2psi[f]);
+    for (int a = 0; a < 3; ++a) {
+      const double s = a0[0] * g[a + 1][0] + a0[1] * g[a + 1][1] + a0[2] * g[a + 1][2];
+      const double ys = Vm * s, rs = cr * s;
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const double bh = sa * Af[f][i] - I4[f] / 3.0 * h[a][i];  // beta_f h_a
-        P[a][i] += cw * (bh + sa * Af[f][i]);
-        r[f][a][i] = cr * bh;
+        y[a][i] += ys * A[i];
+        r[f][a][i] = rs * A[i] - ch * h[a][i];
       }
     }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      P[a][i] *= V;
-      Pv[a][i] = P[a][i] + V * c11 * h[a][i];
-    }
   }
-  // diagonal-in-(i,j) part: D_ab = V ((c_Q/2) h_a.h_b + h_a.tau h_b)
-  const double hq = 0.5 * cQ * V;
-  double* Kout = Ke + (size_t)e * ke_packed(12);
+  w *= 1.0 / 3.0;
+  const double T = V * (kappa * (J - 1.0) * J - w);
+  const double bt = V * (0.5 * kappa * (2.0 * J - 1.0) * J + w * (1.0 / 3.0));
+  if (fe) {
+    double f0[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = a; b < 4; ++b) {
-      const double D = hq * (h[a][0] * h[b][0] + h[a][1] * h[b][1] + h[a][2] * h[b][2]) +
-                       V * (h[a][0] * th[b][0] + h[a][1] * th[b][1] + h[a][2] * th[b][2]);
+      for (int i = 0; i < 3; ++i) {
+        const double v = y[a][i] + T * h[a][i];
+        fe[(size_t)e * 12 + 3 * (a + 1) + i] = v;
+        f0[i] -= v;
+      }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) fe[(size_t)e * 12 + i] = f0[i];
+  }
+  double p[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) p[a][i] = bt * h[a][i] - (2.0 / 3.0) * y[a][i];
+  // block rows 1..3 in order (blocks below the diagonal are transposes of
+  // earlier ones), each with its node-0 block; block row 0 last
+  const Out out{Ke + (size_t)e * Out::kStride};
+  double K[3][3][3][3], K0[3][3][3];  // K[a][b][i][j], a <= b; K0[a] = K[a, node 0]
+  auto entry = [&](int a, int b, int i, int j, double D) {
+    double v = p[a][i] * h[b][j] + (i == j ? D : 0.0);
+    v += h[a][i] * p[b][j];
+    v -= T * h[a][j] * h[b][i];
+    v += r[0][a][i] * r[0][b][j];
+    v += r[1][a][i] * r[1][b][j];
+    return v;
+  };
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+#pragma unroll
+    for (int b = a; b < 3; ++b) {
+      const double D = h[a][0] * y[b][0] + h[a][1] * y[b][1] + h[a][2] * y[b][2];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          if (a == b && j < i) continue;
-          double v = Pv[a][i] * h[b][j] + h[a][i] * P[b][j] + hq * h[a][j] * h[b][i] + r[0][a][i] * r[0][b][j] +
-                     r[1][a][i] * r[1][b][j];
-          if (i == j) v += D;
-          Kout[ke_idx(12, 3 * a + i, 3 * b + j)] = v;
-        }
+        for (int j = 0; j < 3; ++j)
+          K[a][b][i][j] = (a == b && j < i) ? K[a][b][j][i] : entry(a, b, i, j, D);
     }
-  if (fe) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) fe[(size_t)e * 12 + 3 * a + i] = V * th[a][i];
+      for (int j = 0; j < 3; ++j) {
+        double s = 0.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) s -= b < a ? K[b][a][j][i] : K[a][b][i][j];
+        K0[a][i][j] = s;
+      }
+    auto emit = [&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      double v[12];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        v[j] = K0[a][i][j];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) v[3 * (b + 1) + j] = b < a ? K[b][a][j][i] : K[a][b][i][j];
+      }
+      if (a == 0) out.template row<3 + i>(v);
+      else if (a == 1) out.template row<6 + i>(v);
+      else out.template row<9 + i>(v);
+    };
+    emit(std::integral_constant<int, 0>{});
+    emit(std::integral_constant<int, 1>{});
+    emit(std::integral_constant<int, 2>{});
   }
+  auto emit0 = [&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    double v[12];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      // symmetric: entry (j, i) is the one of (i, j), j >= i
+      v[j] = j < i ? -(K0[0][i][j] + K0[1][i][j] + K0[2][i][j]) : -(K0[0][j][i] + K0[1][j][i] + K0[2][j][i]);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) v[3 * (b + 1) + j] = K0[b][j][i];
+    }
+    out.template row<i>(v);
+  };
+  emit0(std::integral_constant<int, 0>{});
+  emit0(std::integral_constant<int, 1>{});
+  emit0(std::integral_constant<int, 2>{});
 }
 
 // ---------------------------------------------------------------------------
@@ -1622,10 +1687,10 @@ void launch_elem_linear(int n_tets, const double* coords, const int32_t* tets, d
 
 void launch_elem_hgo(int n_tets, const double* coords, const int32_t* tets, const double* U,
                      const double* fibres, double c, double k1, double k2, double kappa, double* Ke, double* fe,
-                     int* status, cudaStream_t st) {
+                     bool full, int* status, cudaStream_t st) {
   if (n_tets <= 0) return;
-  k_elem_hgo<<<(n_tets + 63) / 64, 64, 0, st>>>(n_tets, coords, tets, U, fibres, c, k1, k2, kappa, Ke, fe,
-                                                status);
+  auto* k = full ? k_elem_hgo<KeFull> : k_elem_hgo<KePacked>;
+  k<<<(n_tets + 63) / 64, 64, 0, st>>>(n_tets, coords, tets, U, fibres, c, k1, k2, kappa, Ke, fe, status);
 }
 
 void launch_assemble(int P, const SubLayout* lay, const int32_t* sub_elem_ptr, const int32_t* sub_elems,
