@@ -114,8 +114,11 @@ struct feti_ctx {
   int tuned_m = 0;                     // nrhs the block schedules were tuned for
   bool tuned = false;
   float* d_vloc32 = nullptr;
-  int2* d_chunk_gp = nullptr;  // first boundary position and count of each chunk
-  int4* d_pos_tab = nullptr;
+  int4* d_gchunk = nullptr;  // chunks of the single-vector projection (launch_gtv_part)
+  int32_t* d_gchunk_ptr = nullptr;
+  int n_gchunks = 0;
+  int4 *d_pos_tab = nullptr, *d_bt_tab = nullptr;
+  int2* d_row_tab = nullptr;
   int32_t *d_chunk_sub = nullptr, *d_chunk_p0 = nullptr, *d_sub_chunk_ptr = nullptr, *d_col_sub = nullptr;
   double* d_gpart = nullptr;
   int32_t *d_gs_ptr = nullptr, *d_gs_pos = nullptr, *d_dir_dof = nullptr;
@@ -1367,16 +1370,34 @@ feti_status build_decomposition(feti_ctx* ctx) {
   FETI_TRY(upload(ctx, &ctx->d_chunk_sub, chunk_sub));
   FETI_TRY(upload(ctx, &ctx->d_chunk_p0, chunk_p0));
   {
-    std::vector<int2> gp(chunk_sub.size());
-    for (size_t c = 0; c < gp.size(); ++c) {
-      const SubLayout& L = ctx->lay[chunk_sub[c]];
-      gp[c] = make_int2(L.boff + chunk_p0[c], std::min(256, L.nbp + L.k - chunk_p0[c]));
-    }
-    FETI_TRY(upload(ctx, &ctx->d_chunk_gp, gp));
+    // the single-vector projection: at most 1024 positions a chunk (balanced
+    // within the subdomain) where that leaves two chunks per SM, else 256
+    auto cut = [&](int most, std::vector<int4>& ch, std::vector<int32_t>& ptr) {
+      ch.clear();
+      ptr.assign(P + 1, 0);
+      for (int s = 0; s < P; ++s) {
+        const SubLayout& L = ctx->lay[s];
+        const int m = L.k > 0 ? L.nbp + L.k : 0;
+        const int n = (m + most - 1) / most;
+        const int len = n > 0 ? ((m + n - 1) / n + 31) / 32 * 32 : 1;
+        for (int p0 = 0; p0 < m; p0 += len) {
+          const uint64_t o = (uint64_t)(L.roff + (int64_t)(L.nI + p0) * L.k);
+          ch.push_back(make_int4(L.boff + p0, std::min(len, m - p0) | L.k << 16, (int)(uint32_t)o, (int)(uint32_t)(o >> 32)));
+        }
+        ptr[s + 1] = (int32_t)ch.size();
+      }
+    };
+    std::vector<int4> ch;
+    std::vector<int32_t> ptr;
+    cut(1024, ch, ptr);
+    if (ch.size() < 304) cut(256, ch, ptr);
+    ctx->n_gchunks = (int)ch.size();
+    FETI_TRY(upload(ctx, &ctx->d_gchunk, ch));
+    FETI_TRY(upload(ctx, &ctx->d_gchunk_ptr, ptr));
   }
   FETI_TRY(upload(ctx, &ctx->d_sub_chunk_ptr, sub_chunk_ptr));
   FETI_TRY(upload(ctx, &ctx->d_col_sub, col_sub));
-  FETI_TRY(dev_alloc(ctx, &ctx->d_gpart, 6 * (size_t)std::max(ctx->n_chunks, 1)));
+  FETI_TRY(dev_alloc(ctx, &ctx->d_gpart, 6 * (size_t)std::max(ctx->n_gchunks, 1)));
   FETI_TRY(upload(ctx, &ctx->d_gtg_i, gi));
   FETI_TRY(upload(ctx, &ctx->d_gtg_j, gj));
   FETI_TRY(upload(ctx, &ctx->d_gtg_ptr, gptr));
@@ -1492,9 +1513,13 @@ feti_status build_decomposition(feti_ctx* ctx) {
   ctx->maps.bt_sgn = ctx->d_bt_sgn;
   ctx->maps.bpos_sub = ctx->d_bpos_sub;
   FETI_TRY(dev_alloc(ctx, &ctx->d_pos_tab, (size_t)ctx->nb_total));
-  feti::launch_pos_table((int)ctx->nb_total, ctx->d_bpos_sub, ctx->d_lay, ctx->d_pos_tab, ctx->stream);
+  FETI_TRY(dev_alloc(ctx, &ctx->d_bt_tab, (size_t)ctx->nb_total));
+  FETI_TRY(dev_alloc(ctx, &ctx->d_row_tab, (size_t)ctx->n_lambda));
+  feti::launch_map_tables(ctx->maps, ctx->d_lay, ctx->d_pos_tab, ctx->d_bt_tab, ctx->d_row_tab, ctx->stream);
   FETI_CK(cudaGetLastError());
   ctx->maps.pos_tab = ctx->d_pos_tab;
+  ctx->maps.bt_tab = ctx->d_bt_tab;
+  ctx->maps.row_tab = ctx->d_row_tab;
   FETI_CK(cudaStreamSynchronize(ctx->stream));
   return FETI_OK;
 }
@@ -1862,10 +1887,10 @@ void coarse_apply_g(feti_ctx* ctx, const double* g, double* c, const int* done) 
 // d_c = (G^T G)^-1 G^T x from the chunk partials in d_gpart.
 void coarse_apply_part(feti_ctx* ctx, const int* done) {
   if (ctx->coarse_sparse)
-    feti::launch_coarse_solve(ctx->cdag, 1, nullptr, ctx->d_gpart, ctx->d_sub_chunk_ptr, ctx->d_col_sub, ctx->d_lay,
+    feti::launch_coarse_solve(ctx->cdag, 1, nullptr, ctx->d_gpart, ctx->d_gchunk_ptr, ctx->d_col_sub, ctx->d_lay,
                               ctx->d_c, done, ctx->d_coarse_err, ctx->d_spin, ctx->stream);
   else
-    feti::launch_coarse_apply_part((int)ctx->cd, ctx->d_Ginv, ctx->d_gpart, ctx->d_sub_chunk_ptr, ctx->d_col_sub,
+    feti::launch_coarse_apply_part((int)ctx->cd, ctx->d_Ginv, ctx->d_gpart, ctx->d_gchunk_ptr, ctx->d_col_sub,
                                    ctx->d_lay, ctx->d_c, done, ctx->stream);
 }
 
@@ -1880,7 +1905,7 @@ void project(feti_ctx* ctx, const double* v, double* out, const double* a, bool 
     feti::launch_expand(ctx->maps, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
     return;
   }
-  feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_gp, ctx->d_R, ctx->maps, v,
+  feti::launch_gtv_part(ctx->n_gchunks, ctx->d_gchunk, ctx->d_R, ctx->maps, v,
                         ctx->d_gpart, done, st);
   coarse_apply_part(ctx, done);
   feti::launch_expand(ctx->maps, ctx->d_R, v, ctx->d_c, out, a, partial, with_dot, done, st);
@@ -2222,14 +2247,14 @@ void pcg_iteration(feti_ctx* ctx, double* lam, bool f32) {
   local_apply(ctx, 0, ctx->d_p, nullptr, done, f32);                              // q = F p, (p, q)
   feti::launch_scatter(ctx->maps, ctx->d_loc, nullptr, ctx->d_q, ctx->d_p, ctx->d_partial_pq, done, st);
   if (ctx->cd > 0) {
-    feti::launch_gtv_part(ctx->n_chunks, ctx->d_chunk_gp, ctx->d_R, ctx->maps, ctx->d_r, ctx->d_gpart, done, st,
+    feti::launch_gtv_part(ctx->n_gchunks, ctx->d_gchunk, ctx->d_R, ctx->maps, ctx->d_r, ctx->d_gpart, done, st,
                           ctx->d_q, ctx->d_partial_pq, ctx->d_sc, ctx->d_alpha_hist);
     coarse_apply_part(ctx, done);
   }
   feti::launch_expand_update(ctx->maps, ctx->d_R, ctx->d_r, ctx->d_c, ctx->d_w, ctx->d_partial, lam,
                              ctx->d_p, ctx->d_q, ctx->d_partial_pq, ctx->d_sc, ctx->d_alpha_hist, ctx->cd > 0 ? 1 : 0,
                              st);
-  feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, 0, st);
+  feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, nl, 0, st);
 }
 
 feti_status build_pcg_graph(feti_ctx* ctx, int chunk, bool mixed) {
@@ -2353,7 +2378,7 @@ feti_status start_pcg(feti_ctx* ctx, double tol, int maxit) {
   FETI_CK(cudaMemcpyAsync(ctx->d_sc, &h, sizeof(h), cudaMemcpyHostToDevice, ctx->stream));
   FETI_CK(cudaMemsetAsync(ctx->d_p, 0, ctx->n_lambda * sizeof(double), ctx->stream));
   project(ctx, ctx->d_r, ctx->d_w, nullptr, true, &ctx->d_sc->done);
-  feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, 1, ctx->stream);
+  feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, (int)ctx->n_lambda, 1, ctx->stream);
   FETI_CK(cudaGetLastError());
   FETI_CK(cudaMemcpyAsync(ctx->h_sc, ctx->d_sc, sizeof(feti::PcgScalars), cudaMemcpyDeviceToHost, ctx->stream));
   FETI_CK(cudaStreamSynchronize(ctx->stream));

@@ -122,9 +122,13 @@ struct Maps {
   const int32_t* bpos_sub;  // [nb_total] owning subdomain of each boundary position
   const int4* pos_tab;      // [nb_total] kernel dimension, first coarse column and offset of the
                             // R_i row (low, high word) of each boundary position
+  const int4* bt_tab;       // [nb_total] first three rows of each position as 2 row + (sign < 0)
+                            // (-1: none) and the number of further ones
+  const int2* row_tab;      // [n_lambda] the row's positions as 2 pos + (sign < 0), -1: none
 };
-// Fills pos_tab (nb_total entries) from the layouts.
-void launch_pos_table(int nb_total, const int32_t* bpos_sub, const SubLayout* lay, int4* tab, cudaStream_t st);
+// Fills the three tables from the lists and the layouts.
+void launch_map_tables(const Maps& mp, const SubLayout* lay, int4* pos_tab, int4* bt_tab, int2* row_tab,
+                       cudaStream_t st);
 
 // y_b = (B_i^T (wv o x))_b: signed gather onto the boundary positions.
 void launch_gather(const Maps& mp, const double* x, const double* wv, double* y, const int* done,
@@ -157,7 +161,7 @@ struct PcgScalars {
   double rho_slot[2];  // rho of the last two iterations, by parity
 };
 int scatter_partials();  // number of partial sums the row kernels produce
-void launch_ctl_conv(PcgScalars* s, const double* partial, int first, cudaStream_t st);
+void launch_ctl_conv(PcgScalars* s, const double* partial, int n, int first, cudaStream_t st);
 void launch_vsub(int n, const double* a, const double* b, double* out, cudaStream_t st);
 
 // Global displacement by the owner rule.
@@ -237,10 +241,11 @@ void launch_vadd(int n, double* a, const double* b, cudaStream_t st);
 
 namespace feti {
 // G^T x over chunks of 256 boundary positions of the subdomains with k > 0:
-// partial[6 c + a] for chunk c; chunk_gp: first boundary position and count.
+// partial[6 c + a] for chunk c; chunk: first boundary position, count + 2^16 x
+// kernel dimension, offset of its first R row (low, high word).
 // With q != NULL the gathered input is x - alpha q (fused CG update, alpha
 // from the (p, q) partial sums; CTA 0 stores alpha in sc and alpha_hist).
-void launch_gtv_part(int n_chunks, const int2* chunk_gp, const double* R, const Maps& mp, const double* x,
+void launch_gtv_part(int n_chunks, const int4* chunk, const double* R, const Maps& mp, const double* x,
                      double* partial, const int* done, cudaStream_t st, const double* q = nullptr,
                      const double* pq_partial = nullptr, PcgScalars* sc = nullptr, double* alpha_hist = nullptr);
 // Fused CG update + projection expand: r -= alpha q, lam += alpha p in place,

@@ -9,6 +9,7 @@
 #include "feti_internal.h"
 #include "feti_launch.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -37,8 +38,10 @@ __device__ double block_sum(double v, double* red) {
   __syncthreads();
   double t = 0.0;
   if (wid == 0) {
-    t = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.0;
-    t = warp_sum(t);
+    const int nw = (int)(blockDim.x >> 5);
+    t = lane < nw ? red[lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);
   }
   __syncthreads();
   if (threadIdx.x == 0) red[0] = t;
@@ -730,13 +733,6 @@ __global__ void __launch_bounds__(kThreads) k_gemv_loc(const int32_t* __restrict
                                                        const SubLayout* __restrict__ lay, int which,
                                                        const T* __restrict__ M, const T* __restrict__ vloc,
                                                        double* __restrict__ y, const int* __restrict__ done) {
-  dep_wait();
-  dep_go();
-  M = fresh(M);
-  vloc = fresh(vloc);
-  y = fresh(y);
-  done = fresh(done);
-  if (*done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* v = reinterpret_cast<T*>(smem_raw);
   const int s = blk_sub[blockIdx.x];
@@ -745,6 +741,13 @@ __global__ void __launch_bounds__(kThreads) k_gemv_loc(const int32_t* __restrict
   const int m = which == 0 ? L.nbp : L.nbp + L.k;
   constexpr bool f32 = sizeof(T) == 4;
   const int ldm = f32 ? pad4(m) : m;
+  dep_wait();
+  dep_go();
+  M = fresh(M);
+  vloc = fresh(vloc);
+  y = fresh(y);
+  done = fresh(done);
+  if (*done) return;
   const T* Ms = M + (f32 ? (which == 0 ? L.foff32 : L.soff32) : (which == 0 ? L.foff : L.soff));
   for (int p = threadIdx.x; p < ldm; p += blockDim.x) v[p] = p < m ? vloc[L.boff + p] : (T)0;
   if (which == 0 && r0 == 0)
@@ -804,23 +807,91 @@ __global__ void __launch_bounds__(kThreads) k_gemv_loc(const int32_t* __restrict
   }
 }
 
-// Signed gather onto the boundary positions in FP32 (input of the FP32 apply).
-__global__ void k_gather32(Maps mp, const double* __restrict__ x, const double* __restrict__ wv,
-                           float* __restrict__ y, const int* __restrict__ done) {
+// The vector kernels of an iteration are chains of dependent loads (pointer,
+// row, value) around a few FP64 operations.  The topology comes from tables of
+// one 8- or 16-byte entry per row and position, read before the wait for the
+// previous kernel; the values are then loaded at once, and the stop flag after
+// them, so that one memory latency is left.  Newton load step on 32
+// subdomains (6,256 iterations of 14 launches): 600 -> 470 ms; quadratic cube
+// 13.0 -> 12.0 ms.
+//
+// Positions: rows 2 row + (sign < 0) in x, y, z (-1: none), w further rows in
+// the lists.  Rows: the same code for their two positions.
+__device__ __forceinline__ int4 pos_rows(const Maps& mp, int gp) {
+  return gp < mp.nb_total ? __ldg(mp.bt_tab + gp) : make_int4(-1, -1, -1, 0);
+}
+__device__ __forceinline__ int2 row_poss(const Maps& mp, int r) {
+  return r < mp.n_lambda ? __ldg(mp.row_tab + r) : make_int2(-1, -1);
+}
+__device__ __forceinline__ double signed_val(int t, double v) {  // the sign as an integer operation
+  return __hiloint2double(__double2hiint(v) ^ (int)((unsigned)t << 31), __double2loint(v));
+}
+
+// The stop flag, loaded after the loads that precede it in the program.
+__device__ __forceinline__ int flag_now(const int* done) {
+  int d;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(d) : "l"(done) : "memory");
+  return d;
+}
+
+// Signed sum of the rows beyond the third, continued on v.
+template <typename F>
+__device__ __forceinline__ double more_rows(const Maps& mp, int gp, int n, double v, F x) {
+  const int end = mp.bt_ptr[gp + 1];
+  for (int e = end - n; e < end; e += 4) {
+    double t[4], sg[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int ei = min(e + i, end - 1);
+      sg[i] = mp.bt_sgn[ei];
+      t[i] = x(mp.bt_row[ei]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (e + i < end) v += sg[i] * t[i];
+  }
+  return v;
+}
+
+template <typename T>
+__device__ __forceinline__ void gather_body(const Maps& mp, const double* __restrict__ x,
+                                            const double* __restrict__ wv, T* __restrict__ y,
+                                            const int* __restrict__ done) {
+  int gp = blockIdx.x * blockDim.x + threadIdx.x;
+  int4 t = pos_rows(mp, gp);
   dep_wait();
   dep_go();
   x = fresh(x);
   y = fresh(y);
   done = fresh(done);
-  if (*done) return;
-  for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < mp.nb_total; gp += gridDim.x * blockDim.x) {
-    double val = 0.0;
-    for (int e = mp.bt_ptr[gp]; e < mp.bt_ptr[gp + 1]; ++e) {
-      const int row = mp.bt_row[e];
-      val += mp.bt_sgn[e] * x[row] * (wv ? wv[row] : 1.0);
-    }
-    y[gp] = (float)val;
+  auto at = [&](int row) { return wv ? x[row] * wv[row] : x[row]; };
+  double a, b, c;
+  auto load = [&] {
+    a = t.x >= 0 ? at(t.x >> 1) : 0.0;
+    b = t.y >= 0 ? at(t.y >> 1) : 0.0;
+    c = t.z >= 0 ? at(t.z >> 1) : 0.0;
+  };
+  load();
+  if (flag_now(done)) return;
+  while (gp < mp.nb_total) {
+    const int next = gp + gridDim.x * blockDim.x;
+    const int4 tn = pos_rows(mp, next);
+    double val = signed_val(t.x, a);
+    if (t.y >= 0) val += signed_val(t.y, b);
+    if (t.z >= 0) val += signed_val(t.z, c);
+    if (t.w > 0) val = more_rows(mp, gp, t.w, val, at);
+    y[gp] = (T)val;
+    gp = next;
+    t = tn;
+    load();
   }
+}
+
+// Signed gather onto the boundary positions in FP32 (input of the FP32 apply).
+__global__ void __launch_bounds__(kThreads) k_gather32(Maps mp, const double* __restrict__ x,
+                                                       const double* __restrict__ wv, float* __restrict__ y,
+                                                       const int* __restrict__ done) {
+  gather_body(mp, x, wv, y, done);
 }
 
 // Symmetric FP32 local apply y = M v from the lower block-triangle only (half
@@ -1194,28 +1265,18 @@ __global__ void k_vadd(int n, double* __restrict__ a, const double* __restrict__
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] += b[i];
 }
 
-__global__ void k_gather(Maps mp, const double* __restrict__ x, const double* __restrict__ wv,
-                         double* __restrict__ y, const int* __restrict__ done) {
-  dep_wait();
-  dep_go();
-  x = fresh(x);
-  y = fresh(y);
-  done = fresh(done);
-  if (*done) return;
-  for (int gp = blockIdx.x * blockDim.x + threadIdx.x; gp < mp.nb_total; gp += gridDim.x * blockDim.x) {
-    double val = 0.0;
-    for (int e = mp.bt_ptr[gp]; e < mp.bt_ptr[gp + 1]; ++e) {
-      const int row = mp.bt_row[e];
-      val += mp.bt_sgn[e] * x[row] * (wv ? wv[row] : 1.0);
-    }
-    y[gp] = val;
-  }
+__global__ void __launch_bounds__(kThreads) k_gather(Maps mp, const double* __restrict__ x,
+                                                     const double* __restrict__ wv, double* __restrict__ y,
+                                                     const int* __restrict__ done) {
+  gather_body(mp, x, wv, y, done);
 }
 
 __global__ void __launch_bounds__(kThreads) k_scatter(Maps mp, const double* __restrict__ y,
                                                       const double* __restrict__ wv, double* __restrict__ q,
                                                       const double* __restrict__ a, double* __restrict__ partial,
                                                       const int* __restrict__ done) {
+  int r = blockIdx.x * blockDim.x + threadIdx.x;
+  int2 t = row_poss(mp, r);
   dep_wait();
   dep_go();
   y = fresh(y);
@@ -1223,25 +1284,39 @@ __global__ void __launch_bounds__(kThreads) k_scatter(Maps mp, const double* __r
   a = fresh(a);
   partial = fresh(partial);
   done = fresh(done);
-  if (*done) return;
   __shared__ double red[32];
   double dot = 0.0;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < mp.n_lambda; r += gridDim.x * blockDim.x) {
-    double val = 0.0;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int pos = mp.row_pos[2 * r + e];
-      if (pos >= 0) val += mp.row_sgn[2 * r + e] * y[pos];
-    }
-    if (wv) val *= wv[r];
+  double v0, v1, ar, w;
+  auto load = [&] {
+    const bool in = r < mp.n_lambda;
+    v0 = t.x >= 0 ? y[t.x >> 1] : 0.0;
+    v1 = t.y >= 0 ? y[t.y >> 1] : 0.0;
+    ar = in && partial && a ? a[r] : 0.0;
+    w = in && wv ? wv[r] : 1.0;
+  };
+  load();
+  if (flag_now(done)) return;
+  while (r < mp.n_lambda) {
+    const int next = r + gridDim.x * blockDim.x;
+    const int2 tn = row_poss(mp, next);
+    double val = signed_val(t.x, v0);
+    if (t.y >= 0) val += signed_val(t.y, v1);
+    if (wv) val *= w;
     q[r] = val;
-    if (partial) dot += (a ? a[r] : val) * val;
+    if (partial) dot += (a ? ar : val) * val;
+    r = next;
+    t = tn;
+    load();
   }
-  if (partial) {
-    dot = block_sum(dot, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = dot;
+  if (!partial) return;
+  if (blockIdx.x * blockDim.x >= mp.n_lambda) {  // no rows here
+    if (threadIdx.x == 0) partial[blockIdx.x] = 0.0;
+    return;
   }
+  dot = block_sum(dot, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = dot;
 }
+
 
 __global__ void __launch_bounds__(kThreads) k_gtv(const SubLayout* __restrict__ lay, const double* __restrict__ R,
                                                   Maps mp, const double* __restrict__ x, double* __restrict__ g,
@@ -1266,10 +1341,31 @@ __global__ void __launch_bounds__(kThreads) k_gtv(const SubLayout* __restrict__ 
   }
 }
 
-__device__ double reduce_partials(const double* partial, double* red) {
-  double t = 0.0;
-  for (int i = threadIdx.x; i < kPartials; i += blockDim.x) t += partial[i];
-  return block_sum(t, red);
+// Sum of the partial sums of a row kernel over n rows, in fixed order (the CTAs
+// beyond ceil(n / kThreads) have none).  Four warps, one per scheduler, add
+// them up: every CTA of a kernel does this, and an FP64 instruction of a warp
+// takes 65 clocks of its scheduler whatever the lanes hold.
+__device__ double reduce_partials(const double* partial, int n, double* red) {
+  const int np = min(kPartials, (n + kThreads - 1) / kThreads);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int kPer = (kPartials + 127) / 128;
+  __syncthreads();
+  if (wid < 4) {
+    double v[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) v[i] = threadIdx.x + 128 * i < np ? partial[threadIdx.x + 128 * i] : 0.0;
+    double t = v[0];
+#pragma unroll
+    for (int i = 1; i < kPer; ++i)
+      if (wid * 32 + 128 * i < np) t += v[i];
+    if (wid * 32 < np) t = warp_sum(t);
+    if (lane == 0) red[wid] = t;
+  }
+  __syncthreads();
+  double v = red[lane & 3];
+  if (np > 64) v += __shfl_xor_sync(0xffffffffu, v, 2);
+  if (np > 32) v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return __shfl_sync(0xffffffffu, v, 0);
 }
 
 __device__ __forceinline__ int64_t pos_roff(const int4& t) {
@@ -1283,19 +1379,73 @@ __global__ void k_pos_table(int nb_total, const int32_t* __restrict__ bpos_sub, 
     tab[gp] = make_int4(L.k, L.coff, (int)(uint32_t)o, (int)(uint32_t)(o >> 32));
   }
 }
+__global__ void k_row_tables(Maps mp, int4* __restrict__ bt_tab, int2* __restrict__ row_tab) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(mp.nb_total, mp.n_lambda); i += gridDim.x * blockDim.x) {
+    if (i < mp.nb_total) {
+      int c[3] = {-1, -1, -1};
+      const int e0 = mp.bt_ptr[i], e1 = mp.bt_ptr[i + 1];
+      for (int e = 0; e < min(3, e1 - e0); ++e) c[e] = 2 * mp.bt_row[e0 + e] + (mp.bt_sgn[e0 + e] < 0.0 ? 1 : 0);
+      bt_tab[i] = make_int4(c[0], c[1], c[2], max(0, e1 - e0 - 3));
+    }
+    if (i < mp.n_lambda) {
+      int c[2];
+      for (int e = 0; e < 2; ++e) {
+        const int gp = mp.row_pos[2 * i + e];
+        c[e] = gp < 0 ? -1 : 2 * gp + (mp.row_sgn[2 * i + e] < 0.0 ? 1 : 0);
+      }
+      row_tab[i] = make_int2(c[0], c[1]);
+    }
+  }
+}
 
-// G^T x split over chunks of 256 boundary positions (one CTA per chunk,
-// several per subdomain): partial[c*6 + a] = sum over the chunk of
+// G^T x split over chunks of up to kGtvChunk boundary positions of one
+// subdomain (one CTA per chunk): partial[c*6 + a] = sum over the chunk of
 // R_b[p][a] (B^T x)[p].
 // With q != NULL the input is the updated residual x - alpha q, alpha =
 // rho / (p, q) evaluated by every CTA from the partial sums of (p, q) (the
 // fused CG step); CTA 0 records alpha and flags a breakdown.
-__global__ void __launch_bounds__(kThreads) k_gtv_part(const int2* __restrict__ chunk_gp, int n_chunks,
-                                                       const double* __restrict__ R, Maps mp,
-                                                       const double* __restrict__ x, double* __restrict__ partial,
-                                                       const int* __restrict__ done, const double* __restrict__ q,
+//
+// Bound by the FP64 pipe (6 products a position, 9 adds a warp and 35 a CTA to
+// reduce) and, on small decompositions, by its latencies: the host cuts the
+// subdomains into chunks of at most 1024 positions, four per thread, where that
+// leaves two CTAs per SM, and into chunks of 256 elsewhere.  1024 subdomains
+// (1.18 M positions): 81 us with chunks of 256, 41 us.
+__global__ void __launch_bounds__(kThreads) k_gtv_part(const int4* __restrict__ chunk, const double* __restrict__ R,
+                                                       Maps mp, const double* __restrict__ x,
+                                                       double* __restrict__ partial, const int* __restrict__ done,
+                                                       const double* __restrict__ q,
                                                        const double* __restrict__ pq_partial, PcgScalars* sc,
                                                        double* __restrict__ alpha_hist) {
+  const int c = blockIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int4 ch = __ldg(chunk + c);
+  const int count = ch.y & 0xffff, k = ch.y >> 16;
+  const double* Rc = R + pos_roff(ch);
+  const bool wide = k == 6 && (reinterpret_cast<uintptr_t>(Rc) & 15) == 0;
+  int p = threadIdx.x;
+  int4 t;
+  double Rv[6];
+  auto statics = [&] {  // rows and R row of position p
+    t = pos_rows(mp, p < count ? ch.x + p : mp.nb_total);
+#pragma unroll
+    for (int a = 0; a < 6; ++a) Rv[a] = 0.0;
+    if (p < count) {
+      const double* Rr = Rc + (size_t)p * k;
+      if (wide) {
+#pragma unroll
+        for (int a = 0; a < 6; a += 2) {
+          const double2 v = __ldg(reinterpret_cast<const double2*>(Rr + a));
+          Rv[a] = v.x;
+          Rv[a + 1] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int a = 0; a < 6; ++a)
+          if (a < k) Rv[a] = __ldg(Rr + a);
+      }
+    }
+  };
+  statics();
   dep_wait();
   dep_go();
   x = fresh(x);
@@ -1304,11 +1454,23 @@ __global__ void __launch_bounds__(kThreads) k_gtv_part(const int2* __restrict__ 
   q = fresh(q);
   pq_partial = fresh(pq_partial);
   sc = fresh(sc);
-  if (*done) return;
+  double xr[3], qr[3];
+  auto values = [&] {
+    xr[0] = t.x >= 0 ? x[t.x >> 1] : 0.0;
+    xr[1] = t.y >= 0 ? x[t.y >> 1] : 0.0;
+    xr[2] = t.z >= 0 ? x[t.z >> 1] : 0.0;
+    if (q) {
+      qr[0] = t.x >= 0 ? q[t.x >> 1] : 0.0;
+      qr[1] = t.y >= 0 ? q[t.y >> 1] : 0.0;
+      qr[2] = t.z >= 0 ? q[t.z >> 1] : 0.0;
+    }
+  };
+  values();
+  if (flag_now(done)) return;
   __shared__ double red[32];
   double alpha = 0.0;
   if (q) {
-    const double pq = reduce_partials(pq_partial, red);
+    const double pq = reduce_partials(pq_partial, mp.n_lambda, red);
     alpha = sc->rho / pq;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       if (!(pq > 0.0) || !isfinite(pq)) {
@@ -1320,27 +1482,23 @@ __global__ void __launch_bounds__(kThreads) k_gtv_part(const int2* __restrict__ 
       alpha_hist[sc->it] = alpha;
     }
   }
-  // one position per thread (the gathers' load chains run in parallel);
-  // the six coarse columns are reduced by a transposed warp reduction (8
-  // values -> one per lane group in 9 FP64 adds instead of 6 x 5 on GB300's
-  // narrow FP64 pipe) and the eight warps' results summed in warp order
-  const int c = blockIdx.x;
-  if (c >= n_chunks) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int2 ch = __ldg(chunk_gp + c);
+  // the six coarse columns are reduced by a transposed warp reduction (8 values
+  // -> one per lane group in 9 FP64 adds instead of 6 x 5 on GB300's narrow
+  // FP64 pipe) and the eight warps' results summed in warp order
   double v8[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if ((int)threadIdx.x < ch.y) {
-    const int gp = ch.x + threadIdx.x;
-    const int4 tab = __ldg(mp.pos_tab + gp);
-    double val = 0.0;
-    for (int e = mp.bt_ptr[gp]; e < mp.bt_ptr[gp + 1]; ++e) {
-      const int row = mp.bt_row[e];
-      val += mp.bt_sgn[e] * (q ? x[row] - alpha * q[row] : x[row]);
-    }
-    const double* Rr = R + pos_roff(tab);
+  while (p < count) {
+    const int gp = ch.x + p;
+    auto val_of = [&](int s, int i) { return signed_val(s, q ? xr[i] - alpha * qr[i] : xr[i]); };
+    double val = val_of(t.x, 0);
+    if (t.y >= 0) val += val_of(t.y, 1);
+    if (t.z >= 0) val += val_of(t.z, 2);
+    if (t.w > 0)
+      val = more_rows(mp, gp, t.w, val, [&](int row) { return q ? x[row] - alpha * q[row] : x[row]; });
 #pragma unroll
-    for (int a = 0; a < 6; ++a)
-      if (a < tab.x) v8[a] = Rr[a] * val;
+    for (int a = 0; a < 6; ++a) v8[a] += Rv[a] * val;
+    p += kThreads;
+    statics();
+    values();
   }
   // step 16: keep half the values, add the partner's copy of that half
   double v4[4], v2[2], v1;
@@ -1387,32 +1545,60 @@ __global__ void __launch_bounds__(kThreads) k_gtv_part(const int2* __restrict__ 
 
 // c = Ginv g where g is first summed (fixed order) from the chunk partials of
 // k_gtv_part into shared memory by every CTA.
-__global__ void k_coarse_apply_part(int cd, const double* __restrict__ Ginv, const double* __restrict__ partial,
-                                    const int32_t* __restrict__ sub_chunk_ptr, const int32_t* __restrict__ col_sub,
-                                    const SubLayout* __restrict__ lay, double* __restrict__ c,
-                                    const int* __restrict__ done) {
-  dep_wait();
-  dep_go();
-  Ginv = fresh(Ginv);
-  partial = fresh(partial);
-  c = fresh(c);
-  done = fresh(done);
-  if (*done) return;
+__global__ void __launch_bounds__(kThreads) k_coarse_apply_part(
+    int cd, const double* __restrict__ Ginv, const double* __restrict__ partial,
+    const int32_t* __restrict__ sub_chunk_ptr, const int32_t* __restrict__ col_sub, const SubLayout* __restrict__ lay,
+    double* __restrict__ c, const int* __restrict__ done) {
   extern __shared__ double gsh[];
-  for (int j = threadIdx.x; j < cd; j += blockDim.x) {
-    const int s = col_sub[j];
-    const int a = j - lay[s].coff;
-    double t = 0.0;
-    for (int q = sub_chunk_ptr[s]; q < sub_chunk_ptr[s + 1]; ++q) t += partial[6 * q + a];
-    gsh[j] = t;
-  }
-  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  // before the wait: this warp's first row of the inverse (256 columns of it;
+  // complete before the previous kernel began) and the first column's chunks
+  constexpr int kPre = 8;
+  double pre[kPre];
+#pragma unroll
+  for (int i = 0; i < kPre; ++i)
+    pre[i] = warp < cd && lane + 32 * i < cd ? __ldg(Ginv + (size_t)warp * cd + lane + 32 * i) : 0.0;
+  int j = threadIdx.x, a = 0, q0 = 0, q1 = 0;
+  auto chunks = [&] {
+    const int s = __ldg(col_sub + j);
+    a = j - lay[s].coff;
+    q0 = __ldg(sub_chunk_ptr + s);
+    q1 = __ldg(sub_chunk_ptr + s + 1);
+  };
+  if (j < cd) chunks();
+  dep_wait();
+  dep_go();
+  partial = fresh(partial);
+  c = fresh(c);
+  done = fresh(done);
+  while (j < cd) {
+    double t = 0.0;
+    for (int q = q0; q < q1; q += 8) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = q + i < q1 ? partial[6 * (q + i) + a] : 0.0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (q + i < q1) t += v[i];
+    }
+    gsh[j] = t;
+    j += blockDim.x;
+    if (j < cd) chunks();
+  }
+  if (flag_now(done)) return;  // the same for every thread
+  __syncthreads();
   for (int r = warp; r < cd; r += nwarps) {
     double acc = 0.0;
-    for (int j = lane; j < cd; j += 32) acc += Ginv[(size_t)r * cd + j] * gsh[j];
+    if (r == warp) {
+#pragma unroll
+      for (int i = 0; i < kPre; ++i)
+        if (lane + 32 * i < cd) acc += pre[i] * gsh[lane + 32 * i];
+      for (int k = lane + 32 * kPre; k < cd; k += 32) acc += __ldg(Ginv + (size_t)r * cd + k) * gsh[k];
+    } else {
+      for (int k = lane; k < cd; k += 32) acc += __ldg(Ginv + (size_t)r * cd + k) * gsh[k];
+    }
     acc = warp_sum(acc);
     if (lane == 0) c[r] = acc;
   }
@@ -1449,6 +1635,27 @@ __global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const double* __re
                                                      const double* __restrict__ c, double* __restrict__ out,
                                                      const double* __restrict__ a, double* __restrict__ partial,
                                                      int with_dot, const int* __restrict__ done, ExpandUpdate upd) {
+  int r = blockIdx.x * blockDim.x + threadIdx.x;
+  // before the wait: the row's positions and their R rows (complete before the
+  // previous kernel began)
+  const int stride = gridDim.x * blockDim.x;
+  int2 t = row_poss(mp, r), tn = row_poss(mp, r + stride);
+  int4 tab[2], tabn[2];
+  double Rv[2][6];
+  auto tabs_of = [&](int2 tt, int4* to) {
+    to[0] = tt.x >= 0 ? __ldg(mp.pos_tab + (tt.x >> 1)) : make_int4(0, 0, 0, 0);
+    to[1] = tt.y >= 0 ? __ldg(mp.pos_tab + (tt.y >> 1)) : make_int4(0, 0, 0, 0);
+  };
+  tabs_of(t, tab);
+  auto rows_of = [&] {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const double* Rr = R + pos_roff(tab[e]);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) Rv[e][k] = k < tab[e].x ? __ldg(Rr + k) : 0.0;
+    }
+  };
+  rows_of();
   dep_wait();
   dep_go();
   v = fresh(v);
@@ -1463,13 +1670,13 @@ __global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const double* __re
   upd.q = fresh(upd.q);
   upd.pq_partial = fresh(upd.pq_partial);
   upd.sc = fresh(upd.sc);
-  if (*done) return;
   __shared__ double red[32];
   double alpha = 0.0;
   if (upd.r && upd.have_alpha) {
     alpha = upd.sc->alpha;
   } else if (upd.r) {
-    const double pq = reduce_partials(upd.pq_partial, red);
+    if (flag_now(done)) return;
+    const double pq = reduce_partials(upd.pq_partial, mp.n_lambda, red);
     alpha = upd.sc->rho / pq;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       if (!(pq > 0.0) || !isfinite(pq)) {
@@ -1482,40 +1689,58 @@ __global__ void __launch_bounds__(kThreads) k_expand(Maps mp, const double* __re
     }
   }
   double dot = 0.0;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < mp.n_lambda; r += gridDim.x * blockDim.x) {
-    double val;
-    if (upd.r) {
-      val = upd.r[r] - alpha * upd.q[r];
-      upd.r[r] = val;
-      upd.lam[r] += alpha * upd.p[r];
-    } else {
-      val = v[r];
-    }
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int gp = mp.row_pos[2 * r + e];
-      if (gp >= 0) {
-        const int4 tab = __ldg(mp.pos_tab + gp);
-        if (tab.x) {
-          const double* Rr = R + pos_roff(tab);
-          double t = 0.0;
-          if (tab.x == 6) {  // a floating subdomain: all twelve loads at once
-#pragma unroll
-            for (int k = 0; k < 6; ++k) t += Rr[k] * c[tab.y + k];
-          } else {
-            for (int k = 0; k < tab.x; ++k) t += Rr[k] * c[tab.y + k];
-          }
-          val -= mp.row_sgn[2 * r + e] * t;
-        }
+  double val = 0.0, ar = 0.0, qr = 0.0, pr = 0.0, lr = 0.0, cv[2][6];
+  auto load = [&] {
+    if (r < mp.n_lambda) {
+      if (with_dot && a) ar = a[r];
+      val = upd.r ? upd.r[r] : v[r];
+      if (upd.r) {
+        qr = upd.q[r];
+        pr = upd.p[r];
+        lr = upd.lam[r];
       }
     }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) cv[e][k] = k < tab[e].x ? c[tab[e].y + k] : 0.0;
+  };
+  load();
+  if (!(upd.r && !upd.have_alpha) && flag_now(done)) return;
+  while (r < mp.n_lambda) {
+    tabs_of(tn, tabn);  // the tables of the next two rows are on their way during this one
+    const int2 t2 = row_poss(mp, r + 2 * stride);
+    if (upd.r) {
+      val -= alpha * qr;
+      upd.r[r] = val;
+      upd.lam[r] = lr + alpha * pr;
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (tab[e].x) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+          if (k < tab[e].x) s += Rv[e][k] * cv[e][k];
+        val -= signed_val(e == 0 ? t.x : t.y, s);
+      }
     out[r] = val;
-    if (with_dot) dot += (a ? a[r] : val) * val;
+    if (with_dot) dot += (a ? ar : val) * val;
+    r += stride;
+    t = tn;
+    tn = t2;
+    tab[0] = tabn[0];
+    tab[1] = tabn[1];
+    rows_of();
+    load();
   }
-  if (with_dot) {
-    dot = block_sum(dot, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = dot;
+  if (!with_dot) return;
+  if (blockIdx.x * blockDim.x >= mp.n_lambda) {  // no rows here
+    if (threadIdx.x == 0) partial[blockIdx.x] = 0.0;
+    return;
   }
+  dot = block_sum(dot, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = dot;
 }
 
 // G^T G: one CTA per pair block (i, j), thread per entry, rows in fixed order.
@@ -1548,14 +1773,15 @@ __global__ void k_gtg(const int32_t* __restrict__ blk_i, const int32_t* __restri
 
 // ---------------------------------------------------------------------------
 
-__global__ void k_ctl_conv(PcgScalars* s, const double* __restrict__ partial, int first) {
+__global__ void __launch_bounds__(kThreads) k_ctl_conv(PcgScalars* s, const double* __restrict__ partial, int n,
+                                                       int first) {
   dep_wait();
   dep_go();
   s = fresh(s);
   partial = fresh(partial);
   if (s->done) return;
   __shared__ double red[32];
-  const double wn = sqrt(reduce_partials(partial, red));
+  const double wn = sqrt(reduce_partials(partial, n, red));
   if (threadIdx.x == 0) {
     if (first) {
       s->wnorm0 = wn;
@@ -1590,9 +1816,15 @@ __global__ void __launch_bounds__(kThreads) k_axpby_rho(int n, double* __restric
   y = fresh(y);
   s = fresh(s);
   partial = fresh(partial);
-  if (s->done) return;
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double y0 = 0.0, p0 = 0.0;
+  if (i < n) {
+    y0 = y[i];
+    p0 = p[i];
+  }
+  if (flag_now(&s->done)) return;
   __shared__ double red[32];
-  const double rho = reduce_partials(partial, red);
+  const double rho = reduce_partials(partial, n, red);
   const int it = s->it;
   const double beta = it > 0 ? rho / s->rho_slot[(it + 1) & 1] : 0.0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1605,8 +1837,20 @@ __global__ void __launch_bounds__(kThreads) k_axpby_rho(int n, double* __restric
     s->beta = beta;
     beta_hist[it] = beta;
   }
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = it > 0 ? y[i] + beta * p[i] : y[i];
+  if (i < n) p[i] = it > 0 ? y0 + beta * p0 : y0;
+  const int stride = gridDim.x * blockDim.x;
+  for (i += stride; i < n; i += 4 * stride) {
+    double yv[4], pv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = i + k * stride;
+      yv[k] = j < n ? y[j] : 0.0;
+      pv[k] = j < n ? p[j] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k * stride < n) p[i + k * stride] = it > 0 ? yv[k] + beta * pv[k] : yv[k];
+  }
 }
 
 __global__ void k_vsub(int n, const double* a, const double* b, double* out) {
@@ -1800,8 +2044,8 @@ void launch_gtg(int n_blocks, const int32_t* blk_i, const int32_t* blk_j, const 
   k_gtg<<<n_blocks, 64, 0, st>>>(blk_i, blk_j, blk_ptr, blk_rows, lay, R, mp, cd, GtG);
 }
 
-void launch_ctl_conv(PcgScalars* s, const double* partial, int first, cudaStream_t st) {
-  (void)launch_dep(k_ctl_conv, dim3(1), dim3(kThreads), 0, st, s, partial, first);
+void launch_ctl_conv(PcgScalars* s, const double* partial, int n, int first, cudaStream_t st) {
+  (void)launch_dep(k_ctl_conv, dim3(1), dim3(kThreads), 0, st, s, partial, n, first);
 }
 void launch_vsub(int n, const double* a, const double* b, double* out, cudaStream_t st) {
   k_vsub<<<grid_for(n), kThreads, 0, st>>>(n, a, b, out);
@@ -1917,16 +2161,19 @@ void launch_vadd(int n, double* a, const double* b, cudaStream_t st) {
   k_vadd<<<grid_for(n), kThreads, 0, st>>>(n, a, b);
 }
 
-void launch_gtv_part(int n_chunks, const int2* chunk_gp, const double* R, const Maps& mp, const double* x,
+void launch_gtv_part(int n_chunks, const int4* chunk, const double* R, const Maps& mp, const double* x,
                      double* partial, const int* done, cudaStream_t st, const double* q, const double* pq_partial,
                      PcgScalars* sc, double* alpha_hist) {
   if (n_chunks <= 0) return;
-  (void)launch_dep(k_gtv_part, dim3(n_chunks), dim3(kThreads), 0, st, chunk_gp, n_chunks, R, mp, x, partial, done, q,
+  (void)launch_dep(k_gtv_part, dim3(n_chunks), dim3(kThreads), 0, st, chunk, R, mp, x, partial, done, q,
                    pq_partial, sc, alpha_hist);
 }
 
-void launch_pos_table(int nb_total, const int32_t* bpos_sub, const SubLayout* lay, int4* tab, cudaStream_t st) {
-  if (nb_total > 0) k_pos_table<<<grid_for(nb_total), kThreads, 0, st>>>(nb_total, bpos_sub, lay, tab);
+void launch_map_tables(const Maps& mp, const SubLayout* lay, int4* pos_tab, int4* bt_tab, int2* row_tab,
+                       cudaStream_t st) {
+  if (mp.nb_total <= 0) return;
+  k_pos_table<<<grid_for(mp.nb_total), kThreads, 0, st>>>(mp.nb_total, mp.bpos_sub, lay, pos_tab);
+  k_row_tables<<<grid_for(std::max(mp.nb_total, mp.n_lambda)), kThreads, 0, st>>>(mp, bt_tab, row_tab);
 }
 
 void launch_expand_update(const Maps& mp, const double* R, double* r, const double* c, double* out, double* partial,
@@ -1939,7 +2186,7 @@ void launch_expand_update(const Maps& mp, const double* R, double* r, const doub
 
 void launch_axpby_rho(int n, double* p, const double* y, PcgScalars* s, const double* partial, double* beta_hist,
                       cudaStream_t st) {
-  (void)launch_dep(k_axpby_rho, dim3(grid_for(n)), dim3(kThreads), 0, st, n, p, y, s, partial, beta_hist);
+  (void)launch_dep(k_axpby_rho, dim3(std::min(grid_for(n), kPartials)), dim3(kThreads), 0, st, n, p, y, s, partial, beta_hist);
 }
 
 void launch_coarse_apply_part(int cd, const double* Ginv, const double* partial, const int32_t* sub_chunk_ptr,

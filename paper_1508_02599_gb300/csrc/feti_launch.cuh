@@ -1,13 +1,17 @@
 // Launches that start before their predecessor in the stream has ended
 // (programmatic dependent launch).  The kernels of a PCG iteration on small
-// decompositions run 2 to 8 us each, of which about one is the launch and the
+// decompositions run 2 to 8 us each, of which several are the launch and the
 // first instructions: with launch_dep the CTAs of the next kernel are placed
-// while the previous one runs, and wait in dep_wait for its end.
+// while the previous one runs, and wait in dep_wait for its end.  dep_go comes
+// after dep_wait: with it first, the CTAs of several kernels waited at once and
+// a Newton load step took 592 ms instead of 476.
 //
-// A kernel launched this way calls dep_wait before it touches any memory that
-// an earlier kernel writes or reads, then takes its pointers to such memory
-// through fresh(): the compiler may otherwise move a load through a
-// __restrict__ pointer above the wait.
+// Before dep_wait such a kernel reads only what no kernel of the same
+// uninterrupted chain of launches writes (the topology's tables, the R rows and
+// the coarse inverse of the setup); it takes its pointers to all other memory
+// through fresh() after it: the compiler may otherwise move a load through a
+// __restrict__ pointer above the wait.  All its threads wait, so a kernel that
+// has ended implies that everything before it has.
 #pragma once
 #include <cuda_runtime.h>
 
