@@ -114,12 +114,12 @@ struct feti_ctx {
   int tuned_m = 0;                     // nrhs the block schedules were tuned for
   bool tuned = false;
   float* d_vloc32 = nullptr;
-  int4* d_gchunk = nullptr;  // chunks of the single-vector projection (launch_gtv_part)
+  int4* d_gchunk = nullptr;  // chunks of the projection (launch_gtv_part), first of each subdomain
   int32_t* d_gchunk_ptr = nullptr;
   int n_gchunks = 0;
   int4 *d_pos_tab = nullptr, *d_bt_tab = nullptr;
   int2* d_row_tab = nullptr;
-  int32_t *d_chunk_sub = nullptr, *d_chunk_p0 = nullptr, *d_sub_chunk_ptr = nullptr, *d_col_sub = nullptr;
+  int32_t *d_col_sub = nullptr;
   double* d_gpart = nullptr;
   int32_t *d_gs_ptr = nullptr, *d_gs_pos = nullptr, *d_dir_dof = nullptr;
   int32_t *d_gs_gdof = nullptr, *d_elem_gs = nullptr, *d_inc_ptr = nullptr, *d_inc = nullptr;
@@ -131,7 +131,6 @@ struct feti_ctx {
   int n_gs = 0;
   double *d_dU = nullptr, *d_Utrial = nullptr, *d_fl = nullptr;
   std::vector<double> h_partial;
-  int n_chunks = 0;
   int32_t *d_gtg_i = nullptr, *d_gtg_j = nullptr, *d_gtg_ptr = nullptr, *d_gtg_rows = nullptr;
   int n_gtg = 0;
   double *d_GtG = nullptr, *d_Ginv = nullptr, *d_Acoarse = nullptr;
@@ -1312,16 +1311,11 @@ feti_status build_decomposition(feti_ctx* ctx) {
         for (int r0 = 0; r0 < m; r0 += rpcs[t]) { tab_sub[w][t].push_back(s); tab_row[w][t].push_back(r0); }
         if (s == P - 1) ctx->tab_ptr[w][t].push_back((int32_t)tab_sub[w][t].size());
       }
-  // chunks of 256 boundary positions for the projection's G^T v
-  std::vector<int32_t> chunk_sub, chunk_p0, sub_chunk_ptr(P + 1, 0), col_sub(std::max<int64_t>(ctx->cd, 1), 0);
+  std::vector<int32_t> col_sub(std::max<int64_t>(ctx->cd, 1), 0);
   for (int s = 0; s < P; ++s) {
     const SubLayout& L = ctx->lay[s];
-    if (L.k > 0)
-      for (int p0 = 0; p0 < L.nbp + L.k; p0 += 256) { chunk_sub.push_back(s); chunk_p0.push_back(p0); }
-    sub_chunk_ptr[s + 1] = (int32_t)chunk_sub.size();
     for (int a = 0; a < L.k; ++a) col_sub[L.coff + a] = s;
   }
-  ctx->n_chunks = (int)chunk_sub.size();
   hvec<double> Rall(roff);  // every subdomain's n x k block copied below
   par_for(P, 8, [&](int64_t s) { std::copy(Rd[s].begin(), Rd[s].end(), Rall.begin() + ctx->lay[s].roff); });
 
@@ -1367,11 +1361,9 @@ feti_status build_decomposition(feti_ctx* ctx) {
     ctx->cfg32[w] = ctx->tab[w][1];  // R=8, 64 rows per CTA
     ctx->cfg32[w].R = 8;
   }
-  FETI_TRY(upload(ctx, &ctx->d_chunk_sub, chunk_sub));
-  FETI_TRY(upload(ctx, &ctx->d_chunk_p0, chunk_p0));
   {
-    // the single-vector projection: at most 1024 positions a chunk (balanced
-    // within the subdomain) where that leaves two chunks per SM, else 256
+    // chunks of the projection's G^T v: at most 1024 positions (balanced within
+    // the subdomain) where that leaves two chunks per SM, else 256
     auto cut = [&](int most, std::vector<int4>& ch, std::vector<int32_t>& ptr) {
       ch.clear();
       ptr.assign(P + 1, 0);
@@ -1395,7 +1387,6 @@ feti_status build_decomposition(feti_ctx* ctx) {
     FETI_TRY(upload(ctx, &ctx->d_gchunk, ch));
     FETI_TRY(upload(ctx, &ctx->d_gchunk_ptr, ptr));
   }
-  FETI_TRY(upload(ctx, &ctx->d_sub_chunk_ptr, sub_chunk_ptr));
   FETI_TRY(upload(ctx, &ctx->d_col_sub, col_sub));
   FETI_TRY(dev_alloc(ctx, &ctx->d_gpart, 6 * (size_t)std::max(ctx->n_gchunks, 1)));
   FETI_TRY(upload(ctx, &ctx->d_gtg_i, gi));
@@ -1878,7 +1869,7 @@ feti_status coarse_join(feti_ctx* ctx) {
 // c = (G^T G)^-1 g (one vector): dense inverse or sparse sweeps.
 void coarse_apply_g(feti_ctx* ctx, const double* g, double* c, const int* done) {
   if (ctx->coarse_sparse)
-    feti::launch_coarse_solve(ctx->cdag, 1, g, nullptr, ctx->d_sub_chunk_ptr, ctx->d_col_sub, ctx->d_lay, c, done,
+    feti::launch_coarse_solve(ctx->cdag, 1, g, nullptr, ctx->d_gchunk_ptr, ctx->d_col_sub, ctx->d_lay, c, done,
                               ctx->d_coarse_err, ctx->d_spin, ctx->stream);
   else
     feti::launch_coarse_apply((int)ctx->cd, ctx->d_Ginv, g, c, done, ctx->stream);
@@ -2642,7 +2633,7 @@ feti_status alloc_multi(feti_ctx* ctx, int nrhs) {
   FETI_TRY(dev_alloc(ctx, &ctx->dm_part_wy, np));
   FETI_TRY(dev_alloc(ctx, &ctx->dm_part_pq, np));
   FETI_TRY(dev_alloc(ctx, &ctx->dm_part_ww, np));
-  FETI_TRY(dev_alloc(ctx, &ctx->dm_gpart, (size_t)std::max(ctx->n_chunks, 1) * 6 * nrhs));
+  FETI_TRY(dev_alloc(ctx, &ctx->dm_gpart, (size_t)std::max(ctx->n_gchunks, 1) * 6 * nrhs));
   FETI_TRY(dev_alloc(ctx, &ctx->dm_g, (size_t)std::max<int64_t>(ctx->cd, 1) * nrhs));
   FETI_TRY(dev_alloc(ctx, &ctx->dm_c, (size_t)std::max<int64_t>(ctx->cd, 1) * nrhs));
   FETI_TRY(dev_alloc(ctx, &ctx->dm_alpha_hist, (size_t)(ctx->opt.maxit + 2) * feti::kMaxRhs));
@@ -2670,6 +2661,18 @@ void local_apply_m(feti_ctx* ctx, int which, int nrhs, const double* x, const do
                       : (which == 0 ? (const void*)ctx->d_F : (const void*)ctx->d_S);
   void* v = f32 ? (void*)ctx->dm_vloc32 : (void*)ctx->dm_vloc;
   feti::launch_gather_m(ctx->maps, nrhs, x, wv, v, f32 ? 1 : 0, done, st);
+  if (!f32 && ctx->fix64[which]) {
+    // column by column where the fixed-point form beats the plain apply: the
+    // products of the block kernel occupy the FP64 pipe nrhs times as long (128
+    // subdomains, 8 columns: 1.42 ms against 0.78)
+    const int nb = (int)ctx->nb_total;
+    for (int k = 0; k < nrhs; ++k) {
+      feti::launch_col_get(nb, nrhs, k, ctx->dm_vloc, ctx->d_vloc, st);
+      gemv_apply(ctx, which, done, false, nullptr, nullptr);
+      feti::launch_col_set(nb, nrhs, k, 1.0, ctx->d_loc, ctx->dm_loc, st);
+    }
+    return;
+  }
   if (f32 && ctx->tc_m[which])
     feti::launch_gemm_tc(ctx->tab[which][2], ctx->d_lay, which, static_cast<const float*>(M), nrhs,
                          static_cast<const float*>(v), ctx->dm_loc, done, ctx->d_tc_err, ctx->tc_m[which],
@@ -2695,15 +2698,15 @@ void project_m(feti_ctx* ctx, int nrhs, const double* v, double* out, const doub
   const bool coarse = ctx->cd > 0;
   if (coarse) {
     // dense: G^T x partials, their sums, Ginv G; sparse: G^T x partials, then the sweeps
-    feti::launch_project_m(ctx->n_chunks, ctx->d_chunk_sub, ctx->d_chunk_p0, ctx->d_sub_chunk_ptr, ctx->d_col_sub,
-                           ctx->d_lay, ctx->d_R, ctx->maps, nrhs, (int)ctx->cd,
+    feti::launch_project_m(ctx->n_gchunks, ctx->d_gchunk, ctx->d_gchunk_ptr, ctx->d_col_sub, ctx->d_lay, ctx->d_R,
+                           ctx->maps, nrhs, (int)ctx->cd,
                            ctx->coarse_sparse ? nullptr : ctx->d_Ginv, r_upd ? r_upd : v, r_upd ? q : nullptr,
                            ctx->dm_sc, ctx->dm_gpart, ctx->dm_g, ctx->dm_c, done, ctx->stream);
     if (ctx->coarse_sparse)
-      feti::launch_coarse_solve(ctx->cdag, nrhs, nullptr, ctx->dm_gpart, ctx->d_sub_chunk_ptr, ctx->d_col_sub,
+      feti::launch_coarse_solve(ctx->cdag, nrhs, nullptr, ctx->dm_gpart, ctx->d_gchunk_ptr, ctx->d_col_sub,
                                 ctx->d_lay, ctx->dm_c, done, ctx->d_coarse_err, ctx->d_spin, ctx->stream);
   }
-  feti::launch_expand_m(ctx->maps, ctx->d_lay, ctx->d_R, nrhs, coarse ? 1 : 0, v, ctx->dm_c, out, a, partial, r_upd,
+  feti::launch_expand_m(ctx->maps, ctx->d_R, nrhs, coarse ? 1 : 0, v, ctx->dm_c, out, a, partial, r_upd,
                         lam, p, q, ctx->dm_sc, done, ctx->stream);
 }
 

@@ -240,7 +240,7 @@ void launch_vadd(int n, double* a, const double* b, cudaStream_t st);
 }  // namespace feti
 
 namespace feti {
-// G^T x over chunks of 256 boundary positions of the subdomains with k > 0:
+// G^T x over chunks of boundary positions of the subdomains with k > 0:
 // partial[6 c + a] for chunk c; chunk: first boundary position, count + 2^16 x
 // kernel dimension, offset of its first R row (low, high word).
 // With q != NULL the gathered input is x - alpha q (fused CG update, alpha
@@ -418,13 +418,13 @@ void launch_scatter_m(const Maps& mp, int nrhs, const double* y, const double* w
                       double* partial, const int* done, cudaStream_t st);
 // c = (G^T G)^-1 G^T (x - alpha q), q optional (fused CG update); with
 // Ginv == NULL only the chunk partials of G^T (x - alpha q) into gpart.
-void launch_project_m(int n_chunks, const int32_t* chunk_sub, const int32_t* chunk_p0, const int32_t* sub_chunk_ptr,
-                      const int32_t* col_sub, const SubLayout* lay, const double* R, const Maps& mp, int nrhs, int cd,
-                      const double* Ginv, const double* x, const double* q, const PcgScalarsM* sc, double* gpart,
-                      double* g, double* c, const int* done, cudaStream_t st);
-void launch_expand_m(const Maps& mp, const SubLayout* lay, const double* R, int nrhs, int has_coarse, const double* v,
-                     const double* c, double* out, const double* a, double* partial, double* r_upd, double* lam,
-                     const double* p, const double* q, const PcgScalarsM* sc, const int* done, cudaStream_t st);
+void launch_project_m(int n_chunks, const int4* chunk, const int32_t* chunk_ptr, const int32_t* col_sub,
+                      const SubLayout* lay, const double* R, const Maps& mp, int nrhs, int cd, const double* Ginv,
+                      const double* x, const double* q, const PcgScalarsM* sc, double* gpart, double* g, double* c,
+                      const int* done, cudaStream_t st);
+void launch_expand_m(const Maps& mp, const double* R, int nrhs, int has_coarse, const double* v, const double* c,
+                     double* out, const double* a, double* partial, double* r_upd, double* lam, const double* p,
+                     const double* q, const PcgScalarsM* sc, const int* done, cudaStream_t st);
 void launch_axpby_rho_m(int n, int nrhs, double* p, const double* y, PcgScalarsM* s, const double* partial,
                         cudaStream_t st);
 void launch_alpha_m(int nrhs, PcgScalarsM* s, const double* partial, double* alpha_hist, cudaStream_t st);
