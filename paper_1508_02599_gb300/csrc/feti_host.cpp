@@ -1705,10 +1705,9 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, double* S64, float* S32,
   cudaStream_t st = ctx->stream;
   const int s0 = ctx->grp[g], pg = ctx->grp[g + 1] - s0;
   const SubLayout* lw = ctx->d_lay_ws + s0;
-  int64_t elems = 0;
-  for (int s = s0; s < s0 + pg; ++s) elems += (int64_t)ctx->lay[s].ld * ctx->lay[s].ld;
-  cudaError_t e = cudaMemsetAsync(A, 0, (size_t)elems * sizeof(T), st);
-  if (e != cudaSuccess) return e;
+  int max_ld = 0;
+  for (int s = s0; s < s0 + pg; ++s) max_ld = std::max(max_ld, ctx->lay[s].ld);
+  feti::launch_clear_lower(pg, max_ld, lw, A, st);
   feti::launch_assemble(pg, lw, ctx->d_sub_elem_ptr + s0, ctx->d_sub_elems, ctx->d_elem_dense, ctx->d_Ke, ctx->nde,
                         A, st);
   if constexpr (sizeof(T) == 8) {
@@ -1742,7 +1741,7 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, double* S64, float* S32,
         rows[phase][t] = std::max(rows[phase][t], m);
       }
     }
-  e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g],
+  cudaError_t e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g],
                                 Lc ? 1 : 0, A, ctx->d_cholz, ctx->d_status, st);
   if (e != cudaSuccess) return e;
   if (ctx->opt.precond == FETI_PREC_DIRICHLET)

@@ -337,6 +337,10 @@ void launch_extract_tiles(int P, int max_m, const SubLayout* lay, int which, con
                           float* sym32, cudaStream_t st);
 void launch_extract_tiles(int P, int max_m, const SubLayout* lay, int which, const double* A, double* out64,
                           float* out32, float* sym32, cudaStream_t st);
+// Zeroes the lower triangles of the workspace (assembly and elimination use
+// nothing else).
+void launch_clear_lower(int P, int max_ld, const SubLayout* lay, double* A, cudaStream_t st);
+void launch_clear_lower(int P, int max_ld, const SubLayout* lay, float* A, cudaStream_t st);
 // One FP32 correction x (+)= L^-T L^-1 r of the FP32-factor K^+ (L the FP32
 // Cholesky factor of K_rr), the sweeps confined to the interior rows:
 // forward: y_I = L_II^-1 r_I (FP32 into yI, local offsets) and

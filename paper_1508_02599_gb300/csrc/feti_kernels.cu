@@ -490,7 +490,8 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const SubLayout* __restri
   owned_rows(sub_elem_ptr[s], sub_elem_ptr[s + 1], sub_elems, elem_dense, nde, owner, [&](int e, int il, int r, int src) {
     const int row = __shfl_sync(0xffffffffu, r, src);
     const int c = __shfl_sync(0xffffffffu, r, src - il + (lane < nde ? lane : 0));
-    if (lane < nde && c >= 0) A[(size_t)row * L.ld + c] += (T)Ke[(size_t)e * kes + ke_idx(nde, il, lane)];
+    if (lane < nde && c >= 0 && c <= row)  // the elimination reads the lower triangle
+      A[(size_t)row * L.ld + c] += (T)Ke[(size_t)e * kes + ke_idx(nde, il, lane)];
   });
 }
 
