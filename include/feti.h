@@ -128,7 +128,7 @@ typedef struct {
   int32_t precision;   /* FETI_FP64, FETI_MIXED or FETI_MIXED_F32FACTOR */
   double tol;          /* stop when ||P r_k||_2 <= tol ||P r_0||_2 */
   int32_t maxit;       /* PCG iteration limit */
-  int32_t chunk;       /* PCG iterations per CUDA-graph launch (0: default 16) */
+  int32_t chunk;       /* PCG iterations per CUDA-graph launch (0: default 16; the last ones by four) */
   int32_t follower;    /* nonzero: pressure follows the deformed surface (Newton) */
   int32_t n_load_steps;
   double newton_tol;
