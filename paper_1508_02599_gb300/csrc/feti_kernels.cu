@@ -115,71 +115,112 @@ __global__ void k_elem_linear(int n_tets, const double* __restrict__ coords, con
 
 // P2 element (10-node tetrahedron, straight edges; nodes: the vertices, then
 // the midpoints of the edges (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)) for Hooke's
-// law, one warp per element: every lane evaluates the gradients of the
-// barycentric coordinates, then takes node-pair blocks (a, b) = lane, lane +
-// 32, .. of the 10 x 10 block grid and writes their 3 x 3 entries.  The
-// gradients of N_a = L_a (2 L_a - 1) and N_ab = 4 L_a L_b are linear, so the
-// degree-2 Gauss rule (four points (alpha, beta, beta, beta) and permutations,
-// weights 1/4) integrates the stiffness exactly.  p0: the lambda term is
-// carried by a piecewise-constant pressure condensed out of the element
-// (Sec. 3.2, static condensation): lambda V bbar_a,i bbar_b,j with bbar_a the
-// element mean of grad N_a, instead of the integral of lambda g_a,i g_b,j.
-__device__ __forceinline__ void p2_grad(const double gL[4][3], const double Lq[4], int a, double g[3]) {
-  if (a < 4) {
-    const double f = 4.0 * Lq[a] - 1.0;
-    g[0] = f * gL[a][0];
-    g[1] = f * gL[a][1];
-    g[2] = f * gL[a][2];
-    return;
-  }
-  const int ea[6] = {0, 0, 0, 1, 1, 2}, eb[6] = {1, 2, 3, 2, 3, 3};
-  const int u = ea[a - 4], v = eb[a - 4];
-  for (int i = 0; i < 3; ++i) g[i] = 4.0 * (Lq[u] * gL[v][i] + Lq[v] * gL[u][i]);
-}
-
-__global__ void k_elem_linear_p2(int n_tets, const double* __restrict__ coords, const int32_t* __restrict__ tets,
-                                 double E, double nu, int p0, double* __restrict__ Ke, int* status) {
-  const int e = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (e >= n_tets) return;
-  double x[4][3], gL[4][3], V;
-  for (int a = 0; a < 4; ++a) {
-    const int n = tets[10 * (size_t)e + a];
-    for (int i = 0; i < 3; ++i) x[a][i] = coords[3 * (size_t)n + i];
-  }
-  if (!p1_gradients(x, gL, V)) {
-    if (lane == 0) set_status(status, DEV_INVERTED);
-    return;
-  }
-  const double lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu));
-  const double mu = E / (2.0 * (1.0 + nu));
-  const double al = (5.0 + 3.0 * sqrt(5.0)) / 20.0, be = (5.0 - sqrt(5.0)) / 20.0;
-  double* K = Ke + (size_t)e * ke_packed(30);
-  for (int blk = lane; blk < 100; blk += 32) {
-    const int a = blk / 10, b = blk % 10;
-    if (b < a) continue;  // upper triangle of node blocks
-    double k9[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    double ma[3] = {0, 0, 0}, mb[3] = {0, 0, 0};
-    for (int q = 0; q < 4; ++q) {
-      double Lq[4];
-      for (int c = 0; c < 4; ++c) Lq[c] = c == q ? al : be;
-      double ga[3], gb[3];
-      p2_grad(gL, Lq, a, ga);
-      p2_grad(gL, Lq, b, gb);
-      const double gab = ga[0] * gb[0] + ga[1] * gb[1] + ga[2] * gb[2];
-      for (int i = 0; i < 3; ++i) {
-        ma[i] += 0.25 * ga[i];
-        mb[i] += 0.25 * gb[i];
-        for (int j = 0; j < 3; ++j) {
-          double v = mu * ga[j] * gb[i] + (p0 ? 0.0 : lam * ga[i] * gb[j]);
-          if (i == j) v += mu * gab;
-          k9[i][j] += 0.25 * v;
-        }
+// law.  With g_c = grad L_c, grad N_a = (4 L_a - 1) g_a at a vertex and
+// grad N_uv = 4 L_u g_v + 4 L_v g_u at a midpoint, so every 3 x 3 block is a sum
+// of one, two or four of the P1 blocks
+//   B^cd_ij = V (lambda g_ci g_dj + mu (g_cj g_di + delta_ij g_c.g_d))
+// weighted by the means of the products of the coefficients, from
+// <L_c L_d> = (1 + delta_cd) / 20 and <L_c> = 1 / 4: between vertices a and c
+// 0.6 (a = c) or -0.2, between vertex a and the midpoint's other end likewise,
+// between midpoints 0.8 (1 + delta).  p0: the lambda term is carried by a
+// piecewise-constant pressure condensed out of the element (Sec. 3.2, static
+// condensation), lambda V bbar_a,i bbar_b,j with bbar_a the mean of grad N_a: zero
+// at a vertex, g_u + g_v at a midpoint.
+//
+// Bound by the FP64 pipe.  A CTA takes eight elements: a thread per element for
+// the gradients, 18 threads per element for the 144 entries B^cd_ij, then a warp
+// per two elements for the 465 packed entries of each, consecutive ones in
+// consecutive lanes, four products each: about 110 warp instructions an element
+// where quadrature by a warp per element took 1500 (10,368 elements: 774 -> 131
+// us).
+constexpr int kP2Elems = 8;
+__global__ void __launch_bounds__(128) k_elem_linear_p2(int n_tets, const double* __restrict__ coords,
+                                                        const int32_t* __restrict__ tets, double lam, double mu, int p0,
+                                                        double* __restrict__ Ke, int* status) {
+  __shared__ double g_sh[kP2Elems][13];      // gradients of L_0 .. L_3, volume (0: no element)
+  __shared__ double B[kP2Elems][2][144];     // V mu part (p0) or both, V lambda part (p0)
+  const int e0 = blockIdx.x * kP2Elems;
+  if (threadIdx.x < kP2Elems) {
+    const int e = e0 + threadIdx.x;
+    double V = 0.0;
+    if (e < n_tets) {
+      double x[4][3], g[4][3];
+      for (int a = 0; a < 4; ++a) {
+        const int n = tets[10 * (size_t)e + a];
+        for (int i = 0; i < 3; ++i) x[a][i] = coords[3 * (size_t)n + i];
+      }
+      if (p1_gradients(x, g, V)) {
+        for (int a = 0; a < 4; ++a)
+          for (int i = 0; i < 3; ++i) g_sh[threadIdx.x][3 * a + i] = g[a][i];
+      } else {
+        set_status(status, DEV_INVERTED);
+        V = 0.0;
       }
     }
-    for (int i = 0; i < 3; ++i)
-      for (int j = (a == b ? i : 0); j < 3; ++j)
-        K[ke_idx(30, 3 * a + i, 3 * b + j)] = V * (k9[i][j] + (p0 ? lam * ma[i] * mb[j] : 0.0));
+    g_sh[threadIdx.x][12] = V;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < kP2Elems * 144; idx += 128) {
+    const int el = idx / 144, q = idx - 144 * el;
+    const int c = q / 36, d = q / 9 % 4, i = q / 3 % 3, j = q % 3;
+    const double* g = g_sh[el];
+    const double V = g[12];
+    if (V == 0.0) continue;
+    double m = g[3 * c + j] * g[3 * d + i];
+    if (i == j) m += g[3 * c] * g[3 * d] + g[3 * c + 1] * g[3 * d + 1] + g[3 * c + 2] * g[3 * d + 2];
+    const double l = lam * g[3 * c + i] * g[3 * d + j];
+    B[el][0][q] = V * (p0 ? mu * m : mu * m + l);
+    B[el][1][q] = V * l;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int t = lane; t < ke_packed(30); t += 32) {
+    // row r, column s of packed entry t
+    int r = 0, first = 0;
+    while (first + 30 - r <= t) first += 30 - r++;
+    const int s = r + t - first;
+    const int a = r / 3, b = s / 3, ij = 3 * (r % 3) + s % 3;
+    // ends of the two nodes' edges (a vertex: itself twice)
+    auto ends = [](int n, int& u, int& v) {
+      const int k = n - 4;
+      u = n < 4 ? n : (k < 3 ? 0 : (k < 5 ? 1 : 2));
+      v = n < 4 ? n : (k < 3 ? k + 1 : (k < 5 ? k - 1 : 3));
+    };
+    int u, v, p, q;
+    ends(a, u, v);
+    ends(b, p, q);
+    int o[4] = {0, 0, 0, 0};
+    double w[4] = {0, 0, 0, 0};
+    if (b < 4) {  // two vertices
+      o[0] = 4 * a + b;
+      w[0] = a == b ? 0.6 : -0.2;
+    } else if (a < 4) {  // vertex, midpoint
+      o[0] = 4 * a + q;
+      w[0] = a == p ? 0.6 : -0.2;
+      o[1] = 4 * a + p;
+      w[1] = a == q ? 0.6 : -0.2;
+    } else {
+      o[0] = 4 * v + q;
+      w[0] = u == p ? 1.6 : 0.8;
+      o[1] = 4 * v + p;
+      w[1] = u == q ? 1.6 : 0.8;
+      o[2] = 4 * u + q;
+      w[2] = v == p ? 1.6 : 0.8;
+      o[3] = 4 * u + p;
+      w[3] = v == q ? 1.6 : 0.8;
+    }
+    for (int el = wid; el < kP2Elems; el += 4) {
+      if (g_sh[el][12] == 0.0) continue;
+      const double* Bm = B[el][0] + ij;
+      double k = w[0] * Bm[9 * o[0]];
+#pragma unroll
+      for (int i = 1; i < 4; ++i) k += w[i] * Bm[9 * o[i]];
+      if (p0 && a >= 4) {
+        const double* Bl = B[el][1] + ij;
+        k += (Bl[9 * o[0]] + Bl[9 * o[1]]) + (Bl[9 * o[2]] + Bl[9 * o[3]]);
+      }
+      Ke[(size_t)(e0 + el) * ke_packed(30) + t] = k;
+    }
   }
 }
 
@@ -575,7 +616,7 @@ __global__ void k_augment(const SubLayout* __restrict__ lay, T* __restrict__ Aba
   for (int j = threadIdx.x; j < L.nbp; j += blockDim.x) A[(size_t)(L.n + j) * L.ld + L.nI + j] = (T)1;
 }
 
-// Block sizes of the dense Cholesky kernels: 32-column panels, 64x64 update tiles.
+// Block sizes of the dense coarse elimination: 32-column panels, 64x64 update tiles.
 constexpr int NB = 32;
 constexpr int TT = 64;
 
@@ -1917,8 +1958,8 @@ void launch_face_forces(int n_faces, int fpn, const int32_t* tri, const double* 
 void launch_elem_linear_p2(int n_tets, const double* coords, const int32_t* tets, double E, double nu, int p0,
                            double* Ke, int* status, cudaStream_t st) {
   if (n_tets <= 0) return;
-  const long threads = 32L * n_tets;
-  k_elem_linear_p2<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(n_tets, coords, tets, E, nu, p0, Ke, status);
+  const double lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu)), mu = E / (2.0 * (1.0 + nu));
+  k_elem_linear_p2<<<(n_tets + kP2Elems - 1) / kP2Elems, 128, 0, st>>>(n_tets, coords, tets, lam, mu, p0, Ke, status);
 }
 
 namespace {
