@@ -1,6 +1,6 @@
 """Builds libfeti.so (CUDA kernels + host driver + C ABI) in-tree for sm_103a.
 
-Two translation units compiled in parallel by nvcc, then linked as a shared
+Translation units compiled in parallel by nvcc, then linked as a shared
 library next to this file.  No cmake; the same command works on x86_64 and
 aarch64 hosts.
 """

@@ -1,6 +1,6 @@
-"""The single-vector projection with one chunk per subdomain (more than 304 of
-them, several positions per thread) against the block iteration's, which keeps
-chunks of 256 positions.
+"""The projection with one chunk per subdomain (more than 304 of them, several
+positions per thread) and with chunks of 256 positions, single-vector kernels
+against those of the block iteration.
 
 Both solve to a relative dual residual of 1e-10; with the Dirichlet
 preconditioner the condition number is below 1e3, so the displacements agree to
