@@ -41,9 +41,7 @@ def _compile(src: str, extra: list[str]) -> str:
 def build(verbose_ptxas: bool = False, force: bool = False) -> str:
     """Compile and link; returns the library path.  Rebuilds when sources are newer."""
     os.makedirs(BUILD, exist_ok=True)
-    srcs = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(INCLUDE, "feti.h"),
-                                                      os.path.join(CSRC, "feti_internal.h"), os.path.join(CSRC, "feti_tc.cuh"), os.path.join(CSRC, "feti_fixed.cuh"),
-                                                      os.path.join(CSRC, "feti_launch.cuh"), os.path.join(CSRC, "feti_tables.cuh")]
+    srcs = [os.path.join(INCLUDE, "feti.h")] + [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     if not force and os.path.exists(LIB):
         newest = max(os.path.getmtime(s) for s in srcs)
         if os.path.getmtime(LIB) >= newest:

@@ -19,6 +19,7 @@
 // always drains.  Flags carry an epoch, advanced by the last CTA to finish,
 // so nothing is reset between launches.
 #include "feti_internal.h"
+#include "feti_smem.h"
 
 #include <algorithm>
 
@@ -614,12 +615,11 @@ void launch_coarse_solve(const CoarseDag& dag, int nrhs, const double* g, const 
   if (dag.n_tasks <= 0) return;
   const size_t smem = (size_t)(nrhs == 1 ? dag.smem1 : dag.smem16) * sizeof(double);
   if (nrhs == 1) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_coarse_dag<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)allow_smem(k_coarse_dag<1>, smem);
     k_coarse_dag<1><<<dag.n_tasks, kCT, smem, st>>>(dag, 1, g, partial, sub_chunk_ptr, col_sub, lay, c, done, err,
                                                    spin_cycles);
   } else {
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(k_coarse_dag<kMaxRhs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)allow_smem(k_coarse_dag<kMaxRhs>, smem);
     k_coarse_dag<kMaxRhs><<<dag.n_tasks, kCT, smem, st>>>(dag, nrhs, g, partial, sub_chunk_ptr, col_sub, lay, c,
                                                           done, err, spin_cycles);
   }

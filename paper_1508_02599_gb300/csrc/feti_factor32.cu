@@ -17,6 +17,7 @@
 // block through the explicit F_i (k_kp_fwd_* / k_kp_bwd_*); the FP64
 // residual is an element pass and a row pass (k_elem_kx / k_row_resid).
 #include "feti_internal.h"
+#include "feti_smem.h"
 
 #include <algorithm>
 
@@ -564,18 +565,13 @@ void launch_extract_tiles(int P, int max_m, const SubLayout* lay, int which, con
   if (P > 0 && nT > 0) k_extract_tiles<double><<<dim3(nT * (nT + 1) / 2, P), 256, 0, st>>>(lay, which, A, out64, out32, sym32);
 }
 
-template <typename K>
-void kp_smem_attr(K kern, size_t smem) {
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <typename T>
 void kp_forward(int P, const SubLayout* lay, const T* Lc, const double* r, T* yI, T* zb, int max_nr, int max_nI, cudaStream_t st) {
   if (P <= 0) return;
   const size_t smem = (size_t)std::max(max_nr, 1) * sizeof(T);
   const size_t smem_int = (size_t)(std::max(max_nI, 1) + kKB - 1) / kKB * kKB * sizeof(T);
-  kp_smem_attr(k_kp_fwd_interior<T>, smem_int);
-  kp_smem_attr(k_kp_fwd_boundary<T>, smem);
+  (void)allow_smem(k_kp_fwd_interior<T>, smem_int);
+  (void)allow_smem(k_kp_fwd_boundary<T>, smem);
   k_kp_fwd_interior<T><<<P, kT, smem_int, st>>>(lay, Lc, r, yI);
   const int nblk = std::max(1, (max_nr + 31) / 32);
   k_kp_fwd_boundary<T><<<dim3(nblk, P), kT, smem, st>>>(lay, Lc, r, yI, zb);
@@ -588,8 +584,8 @@ void kp_backward(int P, const SubLayout* lay, const T* Lc, T* yI, const double* 
   const size_t smem = (size_t)std::max(max_nr, 1) * sizeof(T);
   const size_t row = (size_t)(std::max(max_nI, 1) + kKB - 1) / kKB * kKB * sizeof(T);
   const int parts = 5 * row <= 200 * 1024 ? 4 : 1;
-  kp_smem_attr(k_kp_bwd_boundary<T>, smem);
-  kp_smem_attr(k_kp_bwd_interior<T>, (1 + parts) * row);
+  (void)allow_smem(k_kp_bwd_boundary<T>, smem);
+  (void)allow_smem(k_kp_bwd_interior<T>, (1 + parts) * row);
   const int nblk = std::max(1, (max_nr + 31) / 32);
   k_kp_bwd_boundary<T><<<dim3(nblk, P), kT, smem, st>>>(lay, Lc, xb, yI);
   k_kp_bwd_interior<T><<<P, kT, (1 + parts) * row, st>>>(lay, Lc, yI, xb, x, init, parts);

@@ -8,6 +8,7 @@
 // subdomain of uneven size is one batch element of a single launch.
 #include "feti_internal.h"
 #include "feti_launch.cuh"
+#include "feti_smem.h"
 #include "feti_tables.cuh"
 
 #include <algorithm>
@@ -2072,7 +2073,7 @@ static void launch_gemv_t(int n_blocks, const int32_t* blk_sub, const int32_t* b
                           int which, const T* M, const T* vloc, double* y, int max_m, const int* done,
                           cudaStream_t st) {
   const size_t smem = (size_t)((max_m + 3) & ~3) * sizeof(T);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k_gemv_loc<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(k_gemv_loc<T, R>, smem);
   (void)launch_dep(k_gemv_loc<T, R>, dim3(n_blocks), dim3(kThreads), smem, st, blk_sub, blk_row0, rpc, lay, which, M, vloc, y, done);
 }
 
@@ -2119,28 +2120,16 @@ void launch_symv_f32(int G, int n_warps, const int32_t* wsub, const int32_t* wpa
 void launch_symv3_f32(int G, int P, const int32_t* order, int max_m, const SubLayout* lay, int which,
                       const float* Msym, const float* vloc, double* y, const int* done, cudaStream_t st) {
   const size_t smem = (size_t)(kThreads / 32 + 1) * (((size_t)max_m + 3) & ~(size_t)3) * sizeof(float);
-  static size_t attr[3] = {0, 0, 0};
-  const int gi = G == 8 ? 0 : (G == 16 ? 1 : 2);
-  if (smem > 48 * 1024 && smem > attr[gi]) {
-    if (G == 8) cudaFuncSetAttribute(k_symv3_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    else if (G == 16) cudaFuncSetAttribute(k_symv3_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    else cudaFuncSetAttribute(k_symv3_f32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr[gi] = smem;
-  }
-  if (G == 8) k_symv3_f32<8><<<P, kThreads, smem, st>>>(order, lay, which, Msym, vloc, y, done);
-  else if (G == 16) k_symv3_f32<16><<<P, kThreads, smem, st>>>(order, lay, which, Msym, vloc, y, done);
-  else k_symv3_f32<32><<<P, kThreads, smem, st>>>(order, lay, which, Msym, vloc, y, done);
+  auto* k = G == 8 ? k_symv3_f32<8> : G == 16 ? k_symv3_f32<16> : k_symv3_f32<32>;
+  (void)allow_smem(k, smem);
+  k<<<P, kThreads, smem, st>>>(order, lay, which, Msym, vloc, y, done);
 }
 
 void launch_symv2_f32(int n_warps, const int32_t* wsub, const int32_t* wpanel, const SubLayout* lay, int which,
                       const float* Msym, const float* vloc, double* y, float* part, const Maps& mp, const int* done,
                       int* err, const unsigned long long* spin_cycles, cudaStream_t st) {
   const size_t smem = (size_t)SYM_WPC * SYM_NS * SYM_STAGE;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_symv2_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
+  (void)allow_smem(k_symv2_f32, smem);
   const int blocks = (n_warps + SYM_WPC - 1) / SYM_WPC;
   k_symv2_f32<<<blocks, SYM_WPC * 32, smem, st>>>(wsub, wpanel, n_warps, lay, which, Msym, vloc, y, part, done, err,
                                                   spin_cycles);
@@ -2188,8 +2177,7 @@ void launch_coarse_apply_part(int cd, const double* Ginv, const double* partial,
                               cudaStream_t st) {
   if (cd <= 0) return;
   const size_t smem = (size_t)cd * sizeof(double);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_coarse_apply_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(k_coarse_apply_part, smem);
   const int warps = cd < 2432 ? cd : 2432;
   (void)launch_dep(k_coarse_apply_part, dim3((warps * 32 + kThreads - 1) / kThreads), dim3(kThreads), smem, st, cd, Ginv, partial,
                                                                                         sub_chunk_ptr, col_sub, lay,

@@ -15,6 +15,7 @@
 // 48.2 ms, with the FP64 residuals column by column.
 #include "feti_internal.h"
 #include "feti_launch.cuh"
+#include "feti_smem.h"
 #include "feti_tables.cuh"
 #include "feti_tc.cuh"
 
@@ -1632,8 +1633,8 @@ void launch_tc5(int ctas_per_sm, const GemvCfg& cfg, const SubLayout* lay, int w
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (n_sm <= 0) n_sm = 1;
-    cudaFuncSetAttribute(k_gemm_tc5<R, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc5_smem(R, Q));
   }
+  (void)allow_smem(k_gemm_tc5<R, Q>, tc5_smem(R, Q));
   const int grid = std::min(cfg.n_blocks, ctas_per_sm * n_sm);
   if (grid > 0)
     k_gemm_tc5<R, Q><<<grid, TC5_THREADS, tc5_smem(R, Q), st>>>(cfg.blk_sub, cfg.blk_row0, cfg.n_blocks, lay, which,
@@ -1651,7 +1652,7 @@ template <typename T, int R>
 void launch_gemm_t(const GemvCfg& cfg, const SubLayout* lay, int which, const T* M, int nrhs, const T* vloc, double* y,
                    int max_m, const int* done, cudaStream_t st) {
   const size_t smem = (size_t)((max_m + 3) & ~3) * nrhs * sizeof(T);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k_gemm_loc<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(k_gemm_loc<T, R>, smem);
   k_gemm_loc<T, R><<<cfg.n_blocks, kThreads, smem, st>>>(cfg.blk_sub, cfg.blk_row0, cfg.rpc, lay, which, M, nrhs, vloc,
                                                         y, done);
 }
@@ -1693,13 +1694,6 @@ void launch_gemm_loc(const GemvCfg& cfg, const SubLayout* lay, int which, const 
 void launch_gemm_tc(const GemvCfg& cfg, const SubLayout* lay, int which, const float* M, int nrhs, const float* vloc,
                     double* y, const int* done, int* err, int variant, const void* tmaps,
                     const unsigned long long* spin_cycles, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-    cudaFuncSetAttribute(k_gemm_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize, TC2_SMEM);
-    cudaFuncSetAttribute(k_gemm_tc3, cudaFuncAttributeMaxDynamicSharedMemorySize, TC3_SMEM);
-    attr = true;
-  }
   if (variant >= 6 && variant <= 8) {
     const CUtensorMap* mp = static_cast<const CUtensorMap*>(tmaps);
     if (variant == 6)  // 3 raw + 2 tail slots, two CTAs per SM
@@ -1711,12 +1705,7 @@ void launch_gemm_tc(const GemvCfg& cfg, const SubLayout* lay, int which, const f
     return;
   }
   if (variant == 4 || variant == 5) {
-    static bool attr4 = false;
-    if (!attr4) {
-      cudaFuncSetAttribute(k_gemm_tc4<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * TC_STAGE + 1024);
-      cudaFuncSetAttribute(k_gemm_tc4<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * TC_STAGE + 1024);
-      attr4 = true;
-    }
+    (void)(variant == 4 ? allow_smem(k_gemm_tc4<3>, 3 * TC_STAGE + 1024) : allow_smem(k_gemm_tc4<2>, 2 * TC_STAGE + 1024));
     const CUtensorMap* mp = static_cast<const CUtensorMap*>(tmaps);
     if (variant == 4)
       k_gemm_tc4<3><<<cfg.n_blocks, kThreads, 3 * TC_STAGE + 1024, st>>>(cfg.blk_sub, cfg.blk_row0, lay, which, mp,
@@ -1724,16 +1713,20 @@ void launch_gemm_tc(const GemvCfg& cfg, const SubLayout* lay, int which, const f
     else
       k_gemm_tc4<2><<<cfg.n_blocks, kThreads, 2 * TC_STAGE + 1024, st>>>(cfg.blk_sub, cfg.blk_row0, lay, which, mp,
                                                                         nrhs, vloc, y, done, err, spin_cycles);
-  } else if (variant == 3)
+  } else if (variant == 3) {
+    (void)allow_smem(k_gemm_tc3, TC3_SMEM);
     k_gemm_tc3<<<cfg.n_blocks, kThreads, TC3_SMEM, st>>>(cfg.blk_sub, cfg.blk_row0, lay, which,
                                                          static_cast<const CUtensorMap*>(tmaps), nrhs, vloc, y, done,
                                                          err);
-  else if (variant == 2)
+  } else if (variant == 2) {
+    (void)allow_smem(k_gemm_tc2, TC2_SMEM);
     k_gemm_tc2<<<cfg.n_blocks, kThreads, TC2_SMEM, st>>>(cfg.blk_sub, cfg.blk_row0, lay, which, M, nrhs, vloc, y, done,
                                                          err);
-  else
+  } else {
+    (void)allow_smem(k_gemm_tc, TC_SMEM);
     k_gemm_tc<<<cfg.n_blocks, kThreads, TC_SMEM, st>>>(cfg.blk_sub, cfg.blk_row0, lay, which, M, nrhs, vloc, y, done,
                                                        err);
+  }
 }
 
 void launch_scatter_m(const Maps& mp, int nrhs, const double* y, const double* wv, double* q, const double* a,

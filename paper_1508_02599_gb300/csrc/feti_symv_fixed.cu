@@ -33,6 +33,7 @@
 #include "feti_internal.h"
 #include "feti_fixed.cuh"
 #include "feti_launch.cuh"
+#include "feti_smem.h"
 
 #include <cooperative_groups.h>
 
@@ -314,8 +315,7 @@ template <int W>
 cudaError_t launch_fix(int C, int P, const int32_t* order, int max_m, const SubLayout* lay, int which, const int2* M,
                        const int* ex, const double* vloc, double* y, const int* done, cudaStream_t st) {
   const size_t sm = fix_smem(max_m, W);
-  cudaError_t e = cudaFuncSetAttribute(k_symv_fix64<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
+  (void)allow_smem(k_symv_fix64<W>, sm);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(P * C));
   cfg.blockDim = dim3(32 * W);
