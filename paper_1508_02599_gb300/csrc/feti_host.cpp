@@ -2248,21 +2248,43 @@ void pcg_iteration(feti_ctx* ctx, double* lam, bool f32) {
   feti::launch_ctl_conv(ctx->d_sc, ctx->d_partial, nl, 0, st);
 }
 
+// Captures what `body` enqueues on the context's stream as *exec.  A launch that
+// is refused leaves the capture valid but the graph without its kernel, so the
+// launches' errors are looked at before the graph is kept; on any error there is
+// no graph and the stream is no longer captured.
+template <typename Body>
+feti_status capture_graph(feti_ctx* ctx, cudaGraphExec_t* exec, Body&& body) {
+  if (*exec) cudaGraphExecDestroy(*exec);
+  *exec = nullptr;
+  FETI_CK(cudaGetLastError());
+  FETI_CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+  const feti_status s = body();
+  const cudaError_t launch = cudaGetLastError();
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
+  const char* what = "graph capture: ";
+  if (launch != cudaSuccess) {
+    e = launch;
+    what = "launch in a captured graph: ";
+  }
+  if (s == FETI_OK && e == cudaSuccess) {
+    e = cudaGraphInstantiate(exec, g, 0);
+    what = "graph instantiate: ";
+    if (e != cudaSuccess) *exec = nullptr;
+  }
+  if (g) cudaGraphDestroy(g);
+  if (s == FETI_OK && e == cudaSuccess) return FETI_OK;
+  (void)cudaGetLastError();
+  return s != FETI_OK ? s : fail(ctx, FETI_ERR_CUDA, std::string(what) + cudaGetErrorString(e));
+}
+
 feti_status build_pcg_graph(feti_ctx* ctx, int slot, int chunk, bool mixed) {
   cudaGraphExec_t& exec = ctx->pcg_graph[slot];
   if (exec && ctx->pcg_graph_chunk[slot] == chunk && ctx->pcg_graph_mixed[slot] == mixed) return FETI_OK;
-  if (exec) {
-    cudaGraphExecDestroy(exec);
-    exec = nullptr;
-  }
-  cudaGraph_t g = nullptr;
-  FETI_CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-  for (int i = 0; i < chunk; ++i) pcg_iteration(ctx, mixed ? ctx->d_dl : ctx->d_lam, mixed);
-  cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
-  if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&exec, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  FETI_TRY(capture_graph(ctx, &exec, [&]() -> feti_status {
+    for (int i = 0; i < chunk; ++i) pcg_iteration(ctx, mixed ? ctx->d_dl : ctx->d_lam, mixed);
+    return FETI_OK;
+  }));
   ctx->pcg_graph_chunk[slot] = chunk;
   ctx->pcg_graph_mixed[slot] = mixed;
   return FETI_OK;
@@ -2761,16 +2783,10 @@ feti_status build_pcgm_graph(feti_ctx* ctx, int slot, int chunk, int nrhs, bool 
   cudaGraphExec_t& exec = ctx->pcgm_graph[slot];
   if (exec && ctx->pcgm_chunk[slot] == chunk && ctx->pcgm_nrhs[slot] == nrhs && ctx->pcgm_mixed[slot] == mixed)
     return FETI_OK;
-  if (exec) cudaGraphExecDestroy(exec);
-  exec = nullptr;
-  cudaGraph_t g = nullptr;
-  FETI_CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-  for (int i = 0; i < chunk; ++i) pcg_iteration_m(ctx, nrhs, mixed ? ctx->dm_dl : ctx->dm_lam, mixed);
-  cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
-  if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&exec, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  FETI_TRY(capture_graph(ctx, &exec, [&]() -> feti_status {
+    for (int i = 0; i < chunk; ++i) pcg_iteration_m(ctx, nrhs, mixed ? ctx->dm_dl : ctx->dm_lam, mixed);
+    return FETI_OK;
+  }));
   ctx->pcgm_chunk[slot] = chunk;
   ctx->pcgm_nrhs[slot] = nrhs;
   ctx->pcgm_mixed[slot] = mixed;
@@ -3538,26 +3554,23 @@ feti_status feti_dual_apply_multi(feti_ctx* ctx, const double* v, double* q, dou
     ctx->dualm_events.assign(2 * (size_t)n_apply + 2, nullptr);
     for (auto& ev : ctx->dualm_events) FETI_CK(cudaEventCreate(&ev));
     const feti::GemvCfg cfg = f32 ? ctx->cfgm32[0] : ctx->cfgm64[0];
-    cudaGraph_t g = nullptr;
-    FETI_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < n_apply; ++i) {
-      void* vl = f32 ? (void*)ctx->dm_vloc32 : (void*)ctx->dm_vloc;
-      feti::launch_gather_m(ctx->maps, nrhs, v, nullptr, vl, f32 ? 1 : 0, zero, st);
-      FETI_CK(cudaEventRecordWithFlags(ctx->dualm_events[2 + 2 * i], st, cudaEventRecordExternal));
-      if (f32 && ctx->tc_m[0])
-        feti::launch_gemm_tc(ctx->tab[0][2], ctx->d_lay, 0, ctx->d_F32, nrhs, static_cast<const float*>(vl), ctx->dm_loc,
-                             zero, ctx->d_tc_err, ctx->tc_m[0], ctx->d_tmap[0], ctx->d_spin, st);
-      else
-        feti::launch_gemm_loc(cfg, ctx->d_lay, 0, f32 ? (const void*)ctx->d_F32 : (const void*)ctx->d_F, f32 ? 1 : 0,
-                              nrhs, vl, ctx->dm_loc, ctx->max_nb, zero, st);
-      FETI_CK(cudaEventRecordWithFlags(ctx->dualm_events[3 + 2 * i], st, cudaEventRecordExternal));
-      feti::launch_scatter_m(ctx->maps, nrhs, ctx->dm_loc, nullptr, q, nullptr, nullptr, zero, st);
-      apply_M_m(ctx, nrhs, q, z, zero, f32);
-    }
-    FETI_CK(cudaStreamEndCapture(st, &g));
-    cudaError_t e = cudaGraphInstantiate(&ctx->dualm_graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    FETI_TRY(capture_graph(ctx, &ctx->dualm_graph, [&]() -> feti_status {
+      for (int i = 0; i < n_apply; ++i) {
+        void* vl = f32 ? (void*)ctx->dm_vloc32 : (void*)ctx->dm_vloc;
+        feti::launch_gather_m(ctx->maps, nrhs, v, nullptr, vl, f32 ? 1 : 0, zero, st);
+        FETI_CK(cudaEventRecordWithFlags(ctx->dualm_events[2 + 2 * i], st, cudaEventRecordExternal));
+        if (f32 && ctx->tc_m[0])
+          feti::launch_gemm_tc(ctx->tab[0][2], ctx->d_lay, 0, ctx->d_F32, nrhs, static_cast<const float*>(vl), ctx->dm_loc,
+                               zero, ctx->d_tc_err, ctx->tc_m[0], ctx->d_tmap[0], ctx->d_spin, st);
+        else
+          feti::launch_gemm_loc(cfg, ctx->d_lay, 0, f32 ? (const void*)ctx->d_F32 : (const void*)ctx->d_F, f32 ? 1 : 0,
+                                nrhs, vl, ctx->dm_loc, ctx->max_nb, zero, st);
+        FETI_CK(cudaEventRecordWithFlags(ctx->dualm_events[3 + 2 * i], st, cudaEventRecordExternal));
+        feti::launch_scatter_m(ctx->maps, nrhs, ctx->dm_loc, nullptr, q, nullptr, nullptr, zero, st);
+        apply_M_m(ctx, nrhs, q, z, zero, f32);
+      }
+      return FETI_OK;
+    }));
     ctx->dualm_v = v;
     ctx->dualm_q = q;
     ctx->dualm_z = z;
@@ -3665,34 +3678,31 @@ feti_status feti_dual_apply(feti_ctx* ctx, const double* v, double* q, double* z
     for (auto& ev : ctx->dual_events) FETI_CK(cudaEventCreate(&ev));
     // The graph brackets every F-gemv launch with event-record nodes so the
     // dominant kernel is timed inside the same run as the whole apply.
-    cudaGraph_t g = nullptr;
-    FETI_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    const bool f32 = f32_ops(ctx);
-    const bool implicit = !f32 && ctx->opt.local_form == 2;
-    for (int i = 0; i < n_apply; ++i) {
-      if (implicit) {
-        // the timed span is the whole implicit local apply (gather, sweeps, boundary take)
+    FETI_TRY(capture_graph(ctx, &ctx->dual_graph, [&]() -> feti_status {
+      const bool f32 = f32_ops(ctx);
+      const bool implicit = !f32 && ctx->opt.local_form == 2;
+      for (int i = 0; i < n_apply; ++i) {
+        if (implicit) {
+          // the timed span is the whole implicit local apply (gather, sweeps, boundary take)
+          FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[2 + 2 * i], st, cudaEventRecordExternal));
+          local_apply(ctx, 0, v, nullptr, zero, false);
+          FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[3 + 2 * i], st, cudaEventRecordExternal));
+          feti::launch_scatter(ctx->maps, ctx->d_loc, nullptr, q, nullptr, nullptr, zero, st);
+          apply_M(ctx, q, z, zero, f32);
+          continue;
+        }
+        if (f32)
+          feti::launch_gather32(ctx->maps, v, nullptr, ctx->d_vloc32, zero, st);
+        else
+          feti::launch_gather(ctx->maps, v, nullptr, ctx->d_vloc, zero, st);
         FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[2 + 2 * i], st, cudaEventRecordExternal));
-        local_apply(ctx, 0, v, nullptr, zero, false);
+        gemv_apply(ctx, 0, zero, f32);
         FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[3 + 2 * i], st, cudaEventRecordExternal));
         feti::launch_scatter(ctx->maps, ctx->d_loc, nullptr, q, nullptr, nullptr, zero, st);
         apply_M(ctx, q, z, zero, f32);
-        continue;
       }
-      if (f32)
-        feti::launch_gather32(ctx->maps, v, nullptr, ctx->d_vloc32, zero, st);
-      else
-        feti::launch_gather(ctx->maps, v, nullptr, ctx->d_vloc, zero, st);
-      FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[2 + 2 * i], st, cudaEventRecordExternal));
-      gemv_apply(ctx, 0, zero, f32);
-      FETI_CK(cudaEventRecordWithFlags(ctx->dual_events[3 + 2 * i], st, cudaEventRecordExternal));
-      feti::launch_scatter(ctx->maps, ctx->d_loc, nullptr, q, nullptr, nullptr, zero, st);
-      apply_M(ctx, q, z, zero, f32);
-    }
-    FETI_CK(cudaStreamEndCapture(st, &g));
-    cudaError_t e = cudaGraphInstantiate(&ctx->dual_graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(ctx, FETI_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+      return FETI_OK;
+    }));
     ctx->dual_v = v;
     ctx->dual_q = q;
     ctx->dual_z = z;

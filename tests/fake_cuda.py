@@ -68,3 +68,12 @@ def solver(lib, monkeypatch, prob, **opt):
     lib.fake_reset()
     with api.FetiSolver(prob, **opt) as s:
         yield s
+
+
+def dual_apply(lib, s, v, q, z, nrhs=1):
+    """feti_dual_apply or feti_dual_apply_multi on host arrays, which are device arrays here."""
+    a = [C.c_void_p(x.ctypes.data) for x in (v, q, z)]
+    if nrhs == 1:
+        s._check(lib.feti_dual_apply(s._ctx, *a, 1, None))
+    else:
+        s._check(lib.feti_dual_apply_multi(s._ctx, *a, nrhs, 1, None))

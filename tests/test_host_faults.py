@@ -1,0 +1,42 @@
+"""Failing runtime calls in the host driver, on a runtime without a device.
+
+The launches do nothing here, so only statuses, graphs and allocations are
+looked at.
+"""
+import numpy as np
+import pytest
+
+import fake_cuda
+from feti_inputs import mesh
+from paper_1508_02599_gb300 import FetiError
+
+CUDA, GRAPHS, FIXED = 11, 0, 2           # a status and two of the fake's counters
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return fake_cuda.load(fake_cuda.build(str(tmp_path_factory.mktemp("fake_cuda"))))
+
+
+def _prob():
+    return mesh.cube_problem(4, (2, 2, 2))
+
+
+@pytest.mark.parametrize("call", ["solve", "solve_multi", "dual_apply", "dual_apply_multi"])
+def test_refused_launch_in_a_capture_leaves_no_graph(lib, monkeypatch, call):
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric="force", maxit=20) as s:
+        s.prepare()
+        n = s.sizes()["n_lambda"]
+        v, q, z = (np.zeros((n, 2)) for _ in range(3))
+        run = {"solve": s.solve, "solve_multi": lambda: s.solve_multi([1.0, 2.0]),
+               "dual_apply": lambda: fake_cuda.dual_apply(lib, s, v, q, z),
+               "dual_apply_multi": lambda: fake_cuda.dual_apply(lib, s, v, q, z, 2)}[call]
+        lib.fake_refuse_in_capture(1)
+        launched, graphs = lib.fake_count(FIXED), lib.fake_count(GRAPHS)
+        with pytest.raises(FetiError) as ei:
+            run()
+        assert ei.value.status == CUDA and "launch in a captured graph" in str(ei.value)
+        assert lib.fake_count(FIXED) > launched and lib.fake_count(GRAPHS) == graphs
+        lib.fake_refuse_in_capture(0)
+        run()                            # captured anew, not replayed
+        assert lib.fake_count(GRAPHS) > graphs
