@@ -337,9 +337,10 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 8 : 4)
 // from the last: x_b = W_b^T t_b, then L[b, j]^T x_b is taken from every column j
 // before the block; then x (+)= x on rows [0, n_I + n_b') (x_b from the F_i
 // apply, FP64 at the boundary offset), and with init x = that correction,
-// zero on the fixing rows.  `parts` threads share a column (4, or 1 where the
-// copies do not fit), each with 64 / parts of a block's rows and its own copy of
-// the subtracted sums, added in a fixed order when the block is reached.
+// zero on the fixing rows.  Four threads (parts = 4) share a column, each with
+// 16 of a block's rows and its own copy of the subtracted sums, added in a fixed
+// order when the block is reached.  Where five interior vectors do not fit shared
+// memory (parts = 0) a thread owns whole columns and subtracts from the one vector.
 template <typename T>
 __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
     k_kp_bwd_interior(const SubLayout* __restrict__ lay, const T* __restrict__ Lbase, const T* __restrict__ yIbase,
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
   const int nI = L.nI, nbp = L.nbp;
   const int nIp = (nI + kKB - 1) / kKB * kKB;
   T* sub = ys + nIp;  // [parts][nIp]
+  const int np = max(parts, 1);
   const int tid = threadIdx.x;
   __shared__ T ts[kKB], ps[4][kKB];
   const int wj = tid & 63, wi = 16 * (tid >> 6);
@@ -369,7 +371,7 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
   for (int i = tid; i < nIp; i += kT) ys[i] = i < nI ? yI[i] : (T)0;
   for (int i = tid; i < parts * nIp; i += kT) sub[i] = (T)0;
   __syncthreads();
-  const int per = kT / parts, col = tid % per, rows = kKB / parts, i0 = (tid / per) * rows;
+  const int per = kT / np, col = tid % per, rows = kKB / np, i0 = (tid / per) * rows;
   T* mine = sub + (size_t)(tid / per) * nIp;
   for (int I0 = nIp - kKB; I0 >= 0; I0 -= kKB) {
     if (tid < kKB) {
@@ -396,7 +398,10 @@ __global__ void __launch_bounds__(kT, sizeof(T) == 4 ? 5 : 3)
 #pragma unroll
         for (int u = 0; u < 16; ++u) t += a[u] * ys[I0 + h + u];
       }
-      mine[j] += t;
+      if (parts)
+        mine[j] += t;
+      else
+        ys[j] -= t;
     }
     __syncthreads();
   }
@@ -583,7 +588,7 @@ void kp_backward(int P, const SubLayout* lay, const T* Lc, T* yI, const double* 
   if (P <= 0) return;
   const size_t smem = (size_t)std::max(max_nr, 1) * sizeof(T);
   const size_t row = (size_t)(std::max(max_nI, 1) + kKB - 1) / kKB * kKB * sizeof(T);
-  const int parts = 5 * row <= 200 * 1024 ? 4 : 1;
+  const int parts = 5 * row <= 200 * 1024 ? 4 : 0;
   (void)allow_smem(k_kp_bwd_boundary<T>, smem);
   (void)allow_smem(k_kp_bwd_interior<T>, (1 + parts) * row);
   const int nblk = std::max(1, (max_nr + 31) / 32);
