@@ -200,6 +200,7 @@ struct feti_ctx {
   int2* d_fix[2] = {nullptr, nullptr};
   int* d_fixexp[2] = {nullptr, nullptr};
   int fix64[2] = {0, 0};
+  bool fix_dropped = false;  // given back for want of memory
   // symmetric FP32 local applies: lower block-triangles, transposed-product
   // partials, work lists, and the load-group size picked by the autotuner
   // per matrix (0: the full-row kernel is used)
@@ -302,14 +303,58 @@ bool f32_ops(const feti_ctx* ctx) { return ctx->opt.precision != FETI_FP64; }
 bool fp64_ops(const feti_ctx* ctx) { return ctx->opt.precision != FETI_MIXED_F32FACTOR; }
 
 template <class T>
-feti_status dev_alloc(feti_ctx* ctx, T** out, size_t count) {
+void dev_free(feti_ctx* ctx, T*& p) {
+  for (size_t i = 0; p && i < ctx->bufs.size(); ++i)
+    if (ctx->bufs[i].p == p) {
+      ctx->bufs[i] = ctx->bufs.back();
+      ctx->bufs.pop_back();
+      cudaFree(p);
+      p = nullptr;
+    }
+  p = nullptr;
+}
+
+// The fixed-point copies of the FP64 operators are a second form of what the
+// context holds anyway: gives them back, with the graphs that name them, and
+// applies the FP64 rows from now on.  False if there were none.
+bool drop_fixed_point(feti_ctx* ctx) {
+  if (!ctx->d_fix[0] && !ctx->d_fix[1]) return false;
+  cudaStreamSynchronize(ctx->stream);
+  for (cudaGraphExec_t* g : {&ctx->pcg_graph[0], &ctx->pcg_graph[1], &ctx->pcgm_graph[0], &ctx->pcgm_graph[1],
+                             &ctx->dual_graph, &ctx->dualm_graph}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+  for (int w = 0; w < 2; ++w) {
+    dev_free(ctx, ctx->d_fix[w]);
+    dev_free(ctx, ctx->d_fixexp[w]);
+    ctx->fix64[w] = 0;
+  }
+  ctx->fix_dropped = true;
+  return true;
+}
+
+// cudaMalloc; where the memory does not suffice, once more without the
+// fixed-point copies.
+cudaError_t device_malloc(feti_ctx* ctx, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_fixed_point(ctx)) {
+    (void)cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
+// spare: what can be done without, gives back nothing else for it
+template <class T>
+feti_status dev_alloc(feti_ctx* ctx, T** out, size_t count, bool spare = false) {
   if (ctx->dry) {
     *out = nullptr;
     return FETI_OK;
   }
   void* p = nullptr;
   const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = spare ? cudaMalloc(&p, bytes) : device_malloc(ctx, &p, bytes);
   if (e != cudaSuccess) {
     ctx->err = std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? FETI_ERR_OOM : FETI_ERR_CUDA;
@@ -1797,7 +1842,7 @@ feti_status coarse_begin(feti_ctx* ctx) {
   }
   if (ctx->coarse_sparse) {
     // supernodal factorization: fronts workspace only until joined
-    cudaError_t e = cudaMalloc(&ctx->coarse_ws[0], std::max<int64_t>(ctx->cplan.ws, 1) * sizeof(double));
+    cudaError_t e = device_malloc(ctx, &ctx->coarse_ws[0], std::max<int64_t>(ctx->cplan.ws, 1) * sizeof(double));
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
       ctx->coarse_ws[0] = nullptr;
@@ -1817,8 +1862,8 @@ feti_status coarse_begin(feti_ctx* ctx) {
     return FETI_OK;
   }
   {
-    cudaError_t e = cudaMalloc(&ctx->coarse_ws[0], cd * cd * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->coarse_ws[1], 4 * cd * cd * sizeof(double));
+    cudaError_t e = device_malloc(ctx, &ctx->coarse_ws[0], cd * cd * sizeof(double));
+    if (e == cudaSuccess) e = device_malloc(ctx, &ctx->coarse_ws[1], 4 * cd * cd * sizeof(double));
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
       for (void*& q : ctx->coarse_ws)
@@ -2050,27 +2095,36 @@ int tab_index(const feti_ctx* ctx, int w, const feti::GemvCfg& c) {
   return 0;
 }
 
+bool find_pick(uint64_t sig, TunedPick* out) {
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  auto it = g_tune_cache.find(sig);
+  if (it == g_tune_cache.end()) return false;
+  *out = it->second;
+  return true;
+}
+
 feti_status autotune(feti_ctx* ctx) {
   const uint64_t sig = tune_signature(ctx);
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune_cache.find(sig);
-    if (it != g_tune_cache.end()) {
-      const TunedPick& tp = it->second;
-      for (int w = 0; w < 2; ++w) {
-        ctx->cfg64[w] = ctx->tab[w][tp.t64[w]];
-        ctx->cfg64[w].R = tp.r64[w];
-        ctx->cfg32[w] = ctx->tab[w][tp.t32[w]];
-        ctx->cfg32[w].R = tp.r32[w];
-        ctx->sym32[w] = tp.sym[w];
-        ctx->fix64[w] = tp.fix[w];
-      }
-      ctx->tuned = true;
-      return FETI_OK;
+  TunedPick tp{};
+  if (find_pick(sig, &tp)) {
+    for (int w = 0; w < 2; ++w) {
+      ctx->cfg64[w] = ctx->tab[w][tp.t64[w]];
+      ctx->cfg64[w].R = tp.r64[w];
+      ctx->cfg32[w] = ctx->tab[w][tp.t32[w]];
+      ctx->cfg32[w].R = tp.r32[w];
+      ctx->sym32[w] = tp.sym[w];
+      ctx->fix64[w] = ctx->d_fix[w] ? tp.fix[w] : 0;
     }
+    ctx->tuned = true;
+    return FETI_OK;
   }
   FETI_TRY(autotune_run(ctx));
-  TunedPick tp{};
+  for (int w = 0; w < 2; ++w)
+    if (!ctx->fix64[w]) {  // the rows are faster
+      dev_free(ctx, ctx->d_fix[w]);
+      dev_free(ctx, ctx->d_fixexp[w]);
+    }
+  if (ctx->fix_dropped) return FETI_OK;  // not the pick of a context that has the memory
   for (int w = 0; w < 2; ++w) {
     tp.t64[w] = tab_index(ctx, w, ctx->cfg64[w]);
     tp.r64[w] = ctx->cfg64[w].R;
@@ -2342,16 +2396,6 @@ feti_status alloc_operators(feti_ctx* ctx) {
       FETI_TRY(dev_alloc(ctx, &ctx->d_kxb, (size_t)ctx->nb_total));
     }
   }
-  // fixed-point copies where the FP64 operators are applied in every
-  // iteration or residual: F_i, and S_i in the FP64 form
-  for (int w = 0; w < 2; ++w) {
-    if (!fp64_ops(ctx) || ctx->opt.per_subdomain || ctx->opt.symmetric == 1 || ctx->sym_max_m[w] <= 0 ||
-        !feti::symv_fixed_fits(ctx->sym_max_m[w]))
-      continue;
-    if (w == 0 ? ctx->opt.local_form == 2 : ctx->opt.precond != FETI_PREC_DIRICHLET || f32_ops(ctx)) continue;
-    FETI_TRY(dev_alloc(ctx, &ctx->d_fix[w], (size_t)ctx->fix_elems[w]));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_fixexp[w], (size_t)ctx->nb_total));
-  }
   if (f32_ops(ctx)) {
     FETI_TRY(dev_alloc(ctx, &ctx->d_F32, (size_t)ctx->op_elems[3]));
     FETI_TRY(dev_alloc(ctx, &ctx->d_S32, (size_t)ctx->op_elems[4]));
@@ -2366,6 +2410,27 @@ feti_status alloc_operators(feti_ctx* ctx) {
   if (ctx->opt.local_form == 2) {
     FETI_TRY(dev_alloc(ctx, &ctx->d_ix, (size_t)ctx->nloc_total));
     FETI_TRY(dev_alloc(ctx, &ctx->d_ix2, (size_t)ctx->nloc_total));
+  }
+  // fixed-point copies where the FP64 operators are applied in every
+  // iteration or residual: F_i, and S_i in the FP64 form.  They come last and may
+  // be missing: half as much again as the FP64 operators (2.7 GB each for 1024
+  // subdomains), and the rows give the same products.
+  TunedPick tp{};
+  const bool known = find_pick(tune_signature(ctx), &tp);
+  for (int w = 0; w < 2; ++w) {
+    if (!fp64_ops(ctx) || ctx->opt.per_subdomain || ctx->opt.symmetric == 1 || ctx->sym_max_m[w] <= 0 ||
+        !feti::symv_fixed_fits(ctx->sym_max_m[w]) || (known && !tp.fix[w]))
+      continue;
+    if (w == 0 ? ctx->opt.local_form == 2 : ctx->opt.precond != FETI_PREC_DIRICHLET || f32_ops(ctx)) continue;
+    feti_status s = dev_alloc(ctx, &ctx->d_fixexp[w], (size_t)ctx->nb_total, true);
+    if (s == FETI_OK) s = dev_alloc(ctx, &ctx->d_fix[w], (size_t)ctx->fix_elems[w], true);
+    if (s == FETI_ERR_OOM) {
+      (void)cudaGetLastError();
+      dev_free(ctx, ctx->d_fixexp[w]);
+      ctx->fix_dropped = true;
+      continue;
+    }
+    FETI_TRY(s);
   }
   return FETI_OK;
 }
@@ -3500,7 +3565,7 @@ feti_status feti_elements(feti_ctx* ctx, const double* U, int32_t u_on_device, d
     FETI_CK(cudaGetLastError());
   } else {
     double* tmp = nullptr;
-    FETI_CK(cudaMalloc(&tmp, std::max<size_t>(full, 1) * sizeof(double)));
+    FETI_CK(device_malloc(ctx, reinterpret_cast<void**>(&tmp), std::max<size_t>(full, 1) * sizeof(double)));
     feti::launch_ke_unpack(ctx->E, ctx->nde, ctx->d_Ke, tmp, st);
     cudaError_t e = cudaMemcpyAsync(Ke_out, tmp, full * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

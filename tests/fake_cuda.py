@@ -57,8 +57,8 @@ def load(path):
         lib = _lib.load(path)
     finally:
         _lib._lib = real
-    lib.fake_live_bytes.restype = C.c_size_t
-    lib.fake_malloc_limit.argtypes = [C.c_size_t, C.c_int]
+    lib.fake_live_bytes.restype = lib.fake_peak_bytes.restype = C.c_size_t
+    lib.fake_capacity.argtypes = [C.c_size_t]
     return lib
 
 

@@ -14,9 +14,7 @@ namespace {
 std::mutex mu;
 cudaError_t last = cudaSuccess;
 std::map<void*, size_t> live;   // device allocations
-size_t live_bytes = 0, largest = 0;
-size_t malloc_above = (size_t)-1;
-int malloc_left = -1;           // allocations above malloc_above that still succeed
+size_t live_bytes = 0, peak_bytes = 0, capacity = (size_t)-1;
 int refuse = 0;                 // 1: launches of the fixed-point apply are refused while a stream is captured
 int capturing = 0, graphs = 0, graph_launches = 0, fixed_launches = 0;
 cudaError_t fail(cudaError_t e) { return last = e; }
@@ -25,14 +23,14 @@ cudaError_t fail(cudaError_t e) { return last = e; }
 extern "C" {
 void fake_reset() {
   last = cudaSuccess;
-  malloc_above = (size_t)-1;
-  malloc_left = -1;
+  capacity = (size_t)-1;
+  peak_bytes = live_bytes;
   refuse = capturing = graphs = graph_launches = fixed_launches = 0;
-  largest = 0;
 }
-void fake_malloc_limit(size_t above, int left) { malloc_above = above, malloc_left = left; }
+void fake_capacity(size_t bytes) { capacity = bytes; }
 void fake_refuse_in_capture(int on) { refuse = on; }
 size_t fake_live_bytes() { return live_bytes; }
+size_t fake_peak_bytes() { return peak_bytes; }
 int fake_count(int what) { return what == 0 ? graphs : what == 1 ? graph_launches : what == 2 ? fixed_launches : capturing; }
 
 
@@ -45,10 +43,11 @@ long fake_fixed_launch() {
 
 cudaError_t cudaMalloc(void** p, size_t n) {
   std::lock_guard<std::mutex> lk(mu);
-  if (n > malloc_above && malloc_left-- <= 0) return fail(cudaErrorMemoryAllocation);
+  if (n > capacity || live_bytes > capacity - n) return fail(cudaErrorMemoryAllocation);
   *p = std::calloc(n ? n : 1, 1);
   live[*p] = n;
   live_bytes += n;
+  if (live_bytes > peak_bytes) peak_bytes = live_bytes;
   return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {

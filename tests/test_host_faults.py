@@ -40,3 +40,52 @@ def test_refused_launch_in_a_capture_leaves_no_graph(lib, monkeypatch, call):
         lib.fake_refuse_in_capture(0)
         run()                            # captured anew, not replayed
         assert lib.fake_count(GRAPHS) > graphs
+
+
+def _prepared_bytes(lib, monkeypatch, symmetric, **opt):
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric=symmetric, maxit=20, **opt) as s:
+        s.prepare()
+        return lib.fake_live_bytes()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_fixed_point_copies_the_tuner_rejects_are_given_back(lib, monkeypatch, precision):
+    """Every launch takes as long here: the rows are kept."""
+    rows = _prepared_bytes(lib, monkeypatch, "off", precision=precision)
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", precision=precision, maxit=20) as s:
+        s.prepare()
+        assert s.schedule()["fp64_F"][0] > 0
+        auto = lib.fake_live_bytes()
+    if precision == "fp64":                # the FP32 forms have further copies beside the full rows
+        assert auto == rows
+        assert _prepared_bytes(lib, monkeypatch, "force") > rows
+    assert _prepared_bytes(lib, monkeypatch, "auto", precision=precision) == auto   # the remembered pick
+
+
+@pytest.mark.parametrize("symmetric", ["auto", "force"])
+def test_memory_for_the_rows_alone_suffices(lib, monkeypatch, symmetric):
+    _prepared_bytes(lib, monkeypatch, "off", workspace_mb=1)
+    need = lib.fake_peak_bytes()
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric=symmetric, workspace_mb=1,
+                          maxit=20) as s:
+        lib.fake_capacity(need)
+        s.prepare()
+        assert s.schedule()["fp64_F"][0] > 0 and s.schedule()["fp64_M"][0] > 0
+        launched = lib.fake_count(FIXED)
+        s.solve()
+        assert lib.fake_count(FIXED) == launched
+
+
+def test_later_allocations_come_before_the_copies(lib, monkeypatch):
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric="force", maxit=20) as s:
+        s.solve()
+        assert s.schedule()["fp64_F"][0] < -400
+        lib.fake_capacity(lib.fake_live_bytes())
+        launched, graphs = lib.fake_count(FIXED), lib.fake_count(GRAPHS)
+        s.solve_multi([1.0, 2.0])          # its vectors fit where the copies were
+        assert s.schedule()["fp64_F"][0] > 0
+        s.solve()                          # not from the graph that names the copies
+        assert lib.fake_count(GRAPHS) >= graphs + 2
+        after = lib.fake_count(FIXED)
+        s.solve()
+        assert lib.fake_count(FIXED) == after and after >= launched
