@@ -201,6 +201,7 @@ struct feti_ctx {
   int* d_fixexp[2] = {nullptr, nullptr};
   int fix64[2] = {0, 0};
   bool fix_dropped = false;  // given back for want of memory
+  bool ops_ready = false;    // every operator array is allocated
   // symmetric FP32 local applies: lower block-triangles, transposed-product
   // partials, work lists, and the load-group size picked by the autotuner
   // per matrix (0: the full-row kernel is used)
@@ -2373,43 +2374,45 @@ double iterations_left(double w_prev, double w, int its, double target) {
 
 // Dense local matrices (factorized in place), S_i, F_i and their FP32 copies.
 feti_status alloc_operators(feti_ctx* ctx) {
-  if (ctx->d_A || ctx->d_A32) return FETI_OK;
-  FETI_TRY(dev_alloc(ctx, &ctx->d_cholz, (size_t)ctx->chol_scratch));
+  if (ctx->ops_ready) return FETI_OK;
+  // what an earlier call got before it ran out of memory is kept
+  auto get = [&](auto** p, size_t n) { return *p ? FETI_OK : dev_alloc(ctx, p, n); };
+  FETI_TRY(get(&ctx->d_cholz, (size_t)ctx->chol_scratch));
   if (f32_factor(ctx)) {
-    FETI_TRY(dev_alloc(ctx, &ctx->d_A32, (size_t)ctx->op_elems[0]));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kr, (size_t)ctx->nloc_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kg, (size_t)ctx->nloc_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_knorm, 2 * (size_t)ctx->P));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kyI, (size_t)ctx->nloc_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kzb, (size_t)ctx->nb_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kxb, (size_t)ctx->nb_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_kye, (size_t)ctx->nde * ctx->E));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_Lc32, (size_t)ctx->lc_elems));
+    FETI_TRY(get(&ctx->d_A32, (size_t)ctx->op_elems[0]));
+    FETI_TRY(get(&ctx->d_kr, (size_t)ctx->nloc_total));
+    FETI_TRY(get(&ctx->d_kg, (size_t)ctx->nloc_total));
+    FETI_TRY(get(&ctx->d_knorm, 2 * (size_t)ctx->P));
+    FETI_TRY(get(&ctx->d_kyI, (size_t)ctx->nloc_total));
+    FETI_TRY(get(&ctx->d_kzb, (size_t)ctx->nb_total));
+    FETI_TRY(get(&ctx->d_kxb, (size_t)ctx->nb_total));
+    FETI_TRY(get(&ctx->d_kye, (size_t)ctx->nde * ctx->E));
+    FETI_TRY(get(&ctx->d_Lc32, (size_t)ctx->lc_elems));
   } else {
-    FETI_TRY(dev_alloc(ctx, &ctx->d_A, (size_t)ctx->op_elems[0]));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_S, (size_t)ctx->op_elems[1]));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_F, (size_t)ctx->op_elems[2]));
+    FETI_TRY(get(&ctx->d_A, (size_t)ctx->op_elems[0]));
+    FETI_TRY(get(&ctx->d_S, (size_t)ctx->op_elems[1]));
+    FETI_TRY(get(&ctx->d_F, (size_t)ctx->op_elems[2]));
     if (!ctx->keep_factor) {
-      FETI_TRY(dev_alloc(ctx, &ctx->d_Lc, (size_t)ctx->lc_elems));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_kyI64, (size_t)ctx->nloc_total));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_kzb64, (size_t)ctx->nb_total));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_kxb, (size_t)ctx->nb_total));
+      FETI_TRY(get(&ctx->d_Lc, (size_t)ctx->lc_elems));
+      FETI_TRY(get(&ctx->d_kyI64, (size_t)ctx->nloc_total));
+      FETI_TRY(get(&ctx->d_kzb64, (size_t)ctx->nb_total));
+      FETI_TRY(get(&ctx->d_kxb, (size_t)ctx->nb_total));
     }
   }
   if (f32_ops(ctx)) {
-    FETI_TRY(dev_alloc(ctx, &ctx->d_F32, (size_t)ctx->op_elems[3]));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_S32, (size_t)ctx->op_elems[4]));
+    FETI_TRY(get(&ctx->d_F32, (size_t)ctx->op_elems[3]));
+    FETI_TRY(get(&ctx->d_S32, (size_t)ctx->op_elems[4]));
     if (ctx->opt.symmetric != 1) {
-      FETI_TRY(dev_alloc(ctx, &ctx->d_F32s, (size_t)ctx->op_elems[5]));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_S32s, (size_t)ctx->op_elems[6]));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_symp, (size_t)ctx->op_elems[7] + 4));
-      FETI_TRY(dev_alloc(ctx, &ctx->d_sym_err, 1));
+      FETI_TRY(get(&ctx->d_F32s, (size_t)ctx->op_elems[5]));
+      FETI_TRY(get(&ctx->d_S32s, (size_t)ctx->op_elems[6]));
+      FETI_TRY(get(&ctx->d_symp, (size_t)ctx->op_elems[7] + 4));
+      FETI_TRY(get(&ctx->d_sym_err, 1));
       FETI_CK(cudaMemsetAsync(ctx->d_sym_err, 0, sizeof(int), ctx->stream));
     }
   }
   if (ctx->opt.local_form == 2) {
-    FETI_TRY(dev_alloc(ctx, &ctx->d_ix, (size_t)ctx->nloc_total));
-    FETI_TRY(dev_alloc(ctx, &ctx->d_ix2, (size_t)ctx->nloc_total));
+    FETI_TRY(get(&ctx->d_ix, (size_t)ctx->nloc_total));
+    FETI_TRY(get(&ctx->d_ix2, (size_t)ctx->nloc_total));
   }
   // fixed-point copies where the FP64 operators are applied in every
   // iteration or residual: F_i, and S_i in the FP64 form.  They come last and may
@@ -2432,6 +2435,7 @@ feti_status alloc_operators(feti_ctx* ctx) {
     }
     FETI_TRY(s);
   }
+  ctx->ops_ready = true;
   return FETI_OK;
 }
 

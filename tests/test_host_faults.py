@@ -10,7 +10,8 @@ import fake_cuda
 from feti_inputs import mesh
 from paper_1508_02599_gb300 import FetiError
 
-CUDA, GRAPHS, FIXED = 11, 0, 2           # a status and two of the fake's counters
+OOM, CUDA = 10, 11                      # statuses
+GRAPHS, FIXED = 0, 2                    # counters of the fake
 
 
 @pytest.fixture(scope="module")
@@ -89,3 +90,18 @@ def test_later_allocations_come_before_the_copies(lib, monkeypatch):
         after = lib.fake_count(FIXED)
         s.solve()
         assert lib.fake_count(FIXED) == after and after >= launched
+
+
+def test_set_up_that_ran_out_of_memory_is_completed_by_the_next(lib, monkeypatch):
+    """No kernel gets an array that the failed set-up did not reach."""
+    full = _prepared_bytes(lib, monkeypatch, "off")
+    with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric="off", maxit=20) as s:
+        base = lib.fake_live_bytes()
+        for part in (0.2, 0.5, 0.8):
+            lib.fake_capacity(int(base + part * (full - base)))
+            with pytest.raises(FetiError) as ei:
+                s.prepare()
+            assert ei.value.status == OOM
+        lib.fake_capacity(2 ** 62)
+        s.prepare()
+        assert lib.fake_live_bytes() == full
