@@ -164,7 +164,10 @@ typedef struct {
                                flight (those drain waits keep a fixed budget of 2e8 clock cycles),
                                releases tensor memory and flags the call, which then returns
                                FETI_ERR_TIMEOUT; the context stays usable.  The same budget bounds
-                               each dependency wait of the sparse coarse solve. */
+                               each dependency wait of the sparse coarse solve, and each wait of the
+                               local factorizations for their copies and tensor-core products; after
+                               a factorization that ran out of it the operators have to be set up
+                               again (feti_prepare or a solve). */
   int32_t coarse_form;      /* the coarse problem (G^T G)^-1 of the projection (Sec. 4.3):
                                0 = automatic (sparse from 1536 coarse columns on), 1 = dense
                                explicit inverse (block elimination; each projection a dense
@@ -424,7 +427,9 @@ feti_status feti_get_refinement(const feti_ctx* ctx, int32_t* steps, double* res
  * later calls on this context, in ns taken literally (100000000 = the default
  * 0.1 s); a budget below one clock cycle, e.g. 0, makes every main-loop wait
  * give up at its first check (the pipelines then always stop, drain and
- * report FETI_ERR_TIMEOUT: a way to exercise that path).  Captured graphs
+ * report FETI_ERR_TIMEOUT: a way to exercise that path); the local
+ * factorizations, which come before them in a solve, keep the default then, and
+ * 1 ns makes them give up too.  Captured graphs
  * read the budget at every launch.  Host blocking: waits for the context's
  * stream. */
 feti_status feti_set_spin_timeout(feti_ctx* ctx, uint64_t spin_timeout_ns);

@@ -156,7 +156,7 @@ struct feti_ctx {
   int *d_status = nullptr, *d_zero = nullptr;
   int *h_status = nullptr;  // pinned
   feti::Maps maps{};
-  bool prepared = false;
+  bool prepared = false, coarse_ready = false;
   // host plan (feti_create_plan): the decomposition without any device state;
   // only the host getters accept it
   bool dry = false;
@@ -219,6 +219,7 @@ struct feti_ctx {
   // main-loop wait budget (SM clock cycles) of the streamed symmetric apply
   // and the warp-specialised tensor-core GEMM: a device word read at every launch
   unsigned long long* d_spin = nullptr;
+  feti::WaitBudget factor_wait{200000, 1000000};
   // FP32-factor form: FP32 elimination workspace (the group workspace, as d_A), per
   // local row its (element, element row) incidences for the FP64 residual of
   // the refined K^+, refinement scratch, per-subdomain norms, and the number
@@ -604,6 +605,13 @@ feti_status set_spin_budget(feti_ctx* ctx, uint64_t ns) {
   const unsigned long long v = cyc > 9.0e18 ? 9000000000000000000ull : (unsigned long long)cyc;
   FETI_CK(cudaMemcpyAsync(ctx->d_spin, &v, sizeof(v), cudaMemcpyHostToDevice, ctx->stream));
   FETI_CK(cudaStreamSynchronize(ctx->stream));
+  // the local factorizations precede the pipelines of a solve that a zero budget
+  // stops: they keep the default then
+  ctx->factor_wait = feti::WaitBudget{200000, 1000000};
+  if (v > 0) {
+    ctx->factor_wait.kcycles = (uint32_t)std::min<unsigned long long>(v >> 10, 1u << 26);
+    ctx->factor_wait.hint_ns = (uint32_t)std::min<uint64_t>(ns, 1000000);
+  }
   return FETI_OK;
 }
 
@@ -1789,12 +1797,12 @@ cudaError_t factorize_group(feti_ctx* ctx, int g, T* A, double* S64, float* S32,
       }
     }
   cudaError_t e = feti::launch_chol_batched(pg, lw, 0, rows[0].data(), (int)rows[0].size(), ctx->d_env0 + ctx->env_off[g],
-                                Lc ? 1 : 0, A, ctx->d_cholz, ctx->d_status, st);
+                                Lc ? 1 : 0, A, ctx->d_cholz, ctx->d_status, ctx->factor_wait, st);
   if (e != cudaSuccess) return e;
   if (ctx->opt.precond == FETI_PREC_DIRICHLET)
     feti::launch_extract_tiles(pg, ctx->max_nb, lw, 0, A, S64, S32, S32s, st);
   e = feti::launch_chol_batched(pg, lw, 1, rows[1].data(), (int)rows[1].size(), nullptr, 0, A, ctx->d_cholz,
-                                ctx->d_status, st);
+                                ctx->d_status, ctx->factor_wait, st);
   if (e != cudaSuccess) return e;
   feti::launch_extract_tiles(pg, ctx->max_nb, lw, 1, A, F64, F32, F32s, st);
   if (Lc) feti::launch_compact_factor(pg, ctx->max_nr, lw, A, Lc, st);
@@ -2446,10 +2454,12 @@ feti_status prepare(feti_ctx* ctx, const double* dU, double tau) {
   lg.mark("setup: allocation");
   FETI_TRY(assemble_all(ctx, dU, tau));
   lg.mark("setup: elements + assembly");
-  if (!ctx->prepared) FETI_TRY(coarse_begin(ctx));
+  ctx->prepared = false;  // a set-up that fails from here on leaves parts of the operators
+  if (!ctx->coarse_ready) FETI_TRY(coarse_begin(ctx));
   feti_status fs = factorize_all(ctx);
   lg.mark("setup: local factorization");
   const feti_status cs = coarse_join(ctx);
+  if (cs == FETI_OK) ctx->coarse_ready = true;
   FETI_TRY(fs);
   FETI_TRY(cs);
   lg.mark("setup: coarse problem (joined)");

@@ -317,13 +317,20 @@ namespace feti {
 // over the subdomains at step t.  winv: store the inverses of the diagonal
 // blocks in place of the blocks (the sweeps over the compact factor multiply
 // by them).  Z: scratch, chol_scratch_bytes per subdomain
-// at SubLayout::zoff.
+// at SubLayout::zoff.  wait: budget of each main-loop wait; one that runs out sets
+// DEV_TIMEOUT.
 constexpr int kCholPanel = 64;
+struct WaitBudget {
+  uint32_t kcycles;  // 1024 SM clock cycles (zero: at the first look)
+  uint32_t hint_ns;  // how long one try may hold its thread
+};
 int64_t chol_scratch_bytes(int n, int elem_bytes);
 cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
-                                const int32_t* env0, int winv, double* A, uint8_t* Z, int* status, cudaStream_t st);
+                                const int32_t* env0, int winv, double* A, uint8_t* Z, int* status,
+                                WaitBudget wait, cudaStream_t st);
 cudaError_t launch_chol_batched(int P, const SubLayout* lay, int phase, const int* step_rows, int n_steps,
-                                const int32_t* env0, int winv, float* A, uint8_t* Z, int* status, cudaStream_t st);
+                                const int32_t* env0, int winv, float* A, uint8_t* Z, int* status,
+                                WaitBudget wait, cudaStream_t st);
 }  // namespace feti
 
 namespace feti {

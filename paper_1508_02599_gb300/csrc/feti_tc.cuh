@@ -22,6 +22,16 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t par) {
   return ok != 0;
 }
 
+// The same, held for hint_ns at most.
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t par, uint32_t hint_ns) {
+  uint32_t ok;
+  asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
+               : "=r"(ok)
+               : "r"(su32(b)), "r"(par), "r"(hint_ns)
+               : "memory");
+  return ok != 0;
+}
+
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes) : "memory");
 }
