@@ -295,8 +295,7 @@ feti_status feti_checkpoint_read(const char* path, double* U, int64_t capacity, 
  * fe_out [n_tets*12] (may be NULL; unused for the linear materials), at the
  * displacement U [n_nodes*3] (NULL = zero).  U and the outputs are host or
  * device pointers as u_on_device / out_on_device say.  Fails with
- * FETI_ERR_ELEMENT_INVERTED if det F <= 0 anywhere (device outputs may then hold
- * part of the results). */
+ * FETI_ERR_ELEMENT_INVERTED if det F <= 0 anywhere, the outputs as they were. */
 feti_status feti_elements(feti_ctx* ctx, const double* U, int32_t u_on_device, double* Ke_out, double* fe_out,
                           int32_t out_on_device);
 
@@ -391,7 +390,9 @@ feti_status feti_kernel_stats(const feti_ctx* ctx, double* gemv_ms, double* gemv
 
 /* Element kernel of the last feti_elements call (the P1 tangent and
  * internal-force kernel of Sec. 3, hyperelastic or linear): its device time
- * (CUDA events on the context's stream around the one launch), the
+ * (CUDA events on the context's stream around it, with the pass over the nodes that
+ * looks for inverted elements before matrices are written straight to a device
+ * array), the
  * algorithmic bytes it must move (connectivity 16 B, fibres 48 B, the
  * symmetric tangent 78 x 8 B, or the full one where it is written straight to a
  * device array, and the force 12 x 8 B per element, coordinates

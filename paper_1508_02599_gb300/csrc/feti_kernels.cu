@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(128) k_elem_linear_p2(int n_tets, const double
 // formed.  The full matrices are written by this kernel as well, a row of 12
 // as three 32-byte stores (whole sectors), instead of being expanded from the
 // packed ones by a second pass.
-struct KeFull {  // row-major 12 x 12, 32-byte aligned
+struct KeFull {  // row-major 12 x 12, 32-byte aligned; only after k_elem_check
+  static constexpr bool kChecked = true;
   static constexpr int kStride = 144;
   double* K;
   template <int r>
@@ -271,6 +272,7 @@ struct KeFull {  // row-major 12 x 12, 32-byte aligned
   }
 };
 struct KePacked {  // upper triangle, 16-byte aligned
+  static constexpr bool kChecked = false;
   static constexpr int kStride = ke_packed(12);
   double* K;
   template <int r>
@@ -287,15 +289,8 @@ struct KePacked {  // upper triangle, 16-byte aligned
   }
 };
 
-template <class Out>
-__global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __restrict__ coords,
-                                                 const int32_t* __restrict__ tets, const double* __restrict__ U,
-                                                 const double* __restrict__ fibres, double cmat, double k1,
-                                                 double k2, double kappa, double* __restrict__ Ke,
-                                                 double* __restrict__ fe, int* status) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n_tets) return;
-  double x[4][3], g[4][3], V, u[4][3];
+__device__ __forceinline__ void load_tet(int e, const double* __restrict__ coords, const int32_t* __restrict__ tets,
+                                         const double* __restrict__ U, double x[4][3], double u[4][3]) {
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
     const int n = tets[4 * e + a];
@@ -305,11 +300,12 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
       u[a][i] = U ? U[3 * n + i] : 0.0;
     }
   }
-  if (!p1_gradients(x, g, V)) {
-    set_status(status, DEV_INVERTED);
-    return;
-  }
-  double F[3][3];
+}
+// Gradients, volume, F, its cofactors cof(F) = J F^-T and J; false where the
+// volume or J is not positive.
+__device__ __forceinline__ bool tet_deformation(const double x[4][3], const double u[4][3], double g[4][3], double& V,
+                                                double F[3][3], double cf[3][3], double& J) {
+  if (!p1_gradients(x, g, V)) return false;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -319,8 +315,6 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
       for (int a = 1; a < 4; ++a) s += (u[a][i] - u[0][i]) * g[a][j];
       F[i][j] = s;
     }
-  // cofactor matrix: cof(F) = J F^-T
-  double cf[3][3];
   cf[0][0] = F[1][1] * F[2][2] - F[1][2] * F[2][1];
   cf[0][1] = F[1][2] * F[2][0] - F[1][0] * F[2][2];
   cf[0][2] = F[1][0] * F[2][1] - F[1][1] * F[2][0];
@@ -330,8 +324,103 @@ __global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __res
   cf[2][0] = F[0][1] * F[1][2] - F[0][2] * F[1][1];
   cf[2][1] = F[0][2] * F[1][0] - F[0][0] * F[1][2];
   cf[2][2] = F[0][0] * F[1][1] - F[0][1] * F[1][0];
-  const double J = F[0][0] * cf[0][0] + F[0][1] * cf[0][1] + F[0][2] * cf[0][2];
-  if (!(J > 0.0)) {
+  J = F[0][0] * cf[0][0] + F[0][1] * cf[0][1] + F[0][2] * cf[0][2];
+  return J > 0.0;
+}
+
+// x truncated to FP32 in integers (zero below its normal range, infinite above).
+__device__ __forceinline__ float trunc_f32(double x) {
+  const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7ff) - 896;
+  const uint32_t m = ((uint32_t)hi & 0xfffff) << 3 | (uint32_t)__double2loint(x) >> 29;
+  const uint32_t v = e <= 0 ? 0u : e >= 255 ? 0x7f800000u : (uint32_t)e << 23 | m;
+  return __uint_as_float(v | ((uint32_t)hi & 0x80000000u));
+}
+__device__ __forceinline__ float det3(const float m[3][3]) {
+  return m[0][0] * (m[1][1] * m[2][2] - m[1][2] * m[2][1]) + m[0][1] * (m[1][2] * m[2][0] - m[1][0] * m[2][2]) +
+         m[0][2] * (m[1][0] * m[2][1] - m[1][1] * m[2][0]);
+}
+// Whether tet_deformation is certain to find both positive, from FP32.  With every
+// coordinate within 2^-20 M = d of its FP32 edge value and edges of at most L the
+// determinants of the edges before and after the deformation are off by less than
+// 18 (L + d)^2 d + 2^-17 (L + d)^3; and where the products of the first add up to
+// at most 2^12 of it, the FP64 J is within 2^-35 of the sum of the products of |F|.
+__device__ __forceinline__ bool surely_positive(const double xd[4][3], const double ud[4][3]) {
+  float E[3][3], D[3][3], A[3][3], M = 0.0f, L = 0.0f;  // edges, their displacements, deformed edges by rows
+  float x0[3], u0[3];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float x = trunc_f32(xd[a][i]), u = trunc_f32(ud[a][i]);
+      M = fmaxf(M, fmaxf(fabsf(x), fabsf(u)));
+      if (a == 0) {
+        x0[i] = x;
+        u0[i] = u;
+        continue;
+      }
+      E[a - 1][i] = x - x0[i];
+      D[a - 1][i] = u - u0[i];
+      A[a - 1][i] = E[a - 1][i] + D[a - 1][i];
+      L = fmaxf(L, fmaxf(fabsf(E[a - 1][i]), fabsf(A[a - 1][i])));
+    }
+  const float d = 0x1p-20f * M, Ld = L + d;
+  const float B = 2.0f * (18.0f * Ld * Ld * d + 0x1p-17f * Ld * Ld * Ld);
+  const float ref = det3(E), def = det3(A);
+  if (!(ref > B && def > B && def < 1e30f && ref < 1e30f)) return false;
+  float G[3][3], Fa[3][3];  // magnitudes: gradients (by node), F
+  float sum = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3, j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+      const float c = fabsf(E[k1][j1] * E[k2][j2]) + fabsf(E[k1][j2] * E[k2][j1]);
+      if (k == 0) sum += fabsf(E[0][j]) * c;
+      G[k][j] = c / ref;
+    }
+  if (!(sum <= 4096.0f * ref)) return false;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      Fa[i][j] = (i == j ? 1.0f : 0.0f) + fabsf(D[0][i]) * G[0][j] + fabsf(D[1][i]) * G[1][j] + fabsf(D[2][i]) * G[2][j];
+  float p = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+    p += Fa[0][j] * (Fa[1][j1] * Fa[2][j2] + Fa[1][j2] * Fa[2][j1]);
+  }
+  return def > 0x1p-24f * p * ref;
+}
+
+// Elements whose volume or det F is not positive, before matrices are written in
+// place: an error leaves the caller's arrays as they were.  In FP32 where that is
+// certain (a pass over the nodes, 200 FP32 operations an element), else by
+// k_elem_hgo's own operations, a sixth of its FP64 time for all of them.
+__global__ void __launch_bounds__(128) k_elem_check(int n_tets, const double* __restrict__ coords,
+                                                    const int32_t* __restrict__ tets, const double* __restrict__ U,
+                                                    int* status) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n_tets) return;
+  double x[4][3], u[4][3];
+  load_tet(e, coords, tets, U, x, u);
+  if (surely_positive(x, u)) return;
+  double g[4][3], V, F[3][3], cf[3][3], J;
+  if (!tet_deformation(x, u, g, V, F, cf, J)) set_status(status, DEV_INVERTED);
+}
+
+template <class Out>
+__global__ void __launch_bounds__(64) k_elem_hgo(int n_tets, const double* __restrict__ coords,
+                                                 const int32_t* __restrict__ tets, const double* __restrict__ U,
+                                                 const double* __restrict__ fibres, double cmat, double k1,
+                                                 double k2, double kappa, double* __restrict__ Ke,
+                                                 double* __restrict__ fe, int* status) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n_tets) return;
+  if (Out::kChecked && *status) return;
+  double x[4][3], g[4][3], V, u[4][3], F[3][3], cf[3][3], J;
+  load_tet(e, coords, tets, U, x, u);
+  if (!tet_deformation(x, u, g, V, F, cf, J)) {
     set_status(status, DEV_INVERTED);
     return;
   }
@@ -1928,6 +2017,7 @@ void launch_elem_hgo(int n_tets, const double* coords, const int32_t* tets, cons
                      const double* fibres, double c, double k1, double k2, double kappa, double* Ke, double* fe,
                      bool full, int* status, cudaStream_t st) {
   if (n_tets <= 0) return;
+  if (full) k_elem_check<<<(n_tets + 127) / 128, 128, 0, st>>>(n_tets, coords, tets, U, status);
   auto* k = full ? k_elem_hgo<KeFull> : k_elem_hgo<KePacked>;
   k<<<(n_tets + 63) / 64, 64, 0, st>>>(n_tets, coords, tets, U, fibres, c, k1, k2, kappa, Ke, fe, status);
 }
