@@ -152,10 +152,16 @@ typedef struct {
                               symmetric kernel (reads only the lower block-triangle of F_i / S_i;
                               FP64: its 56-bit fixed-point copy) when it is faster, 1 = full rows
                               only, 2 = symmetric always (fastest variant; FP64 only while an
-                              operator fits the kernel's shared memory), 3 = symmetric, the FP32
+                              operator fits the kernel's shared memory and the copy the device),
+                              3 = symmetric, the FP32
                               one streamed through shared memory, 4 = symmetric, the FP32 one with
                               one CTA per subdomain (transposed partial sums reduced in shared
-                              memory, no second pass) */
+                              memory, no second pass).  The forms round differently and the pick
+                              is by timing, so results can differ in their last bits between
+                              processes; 1 always gives the same.  FP64 products of m terms by
+                              the copy are within (1.3 m + 80) 2^-48 |M| |v| entry by entry
+                              (rows that it would hold more coarsely are FP64 sums, which are
+                              within m 2^-53), normwise closer than the rows */
   uint64_t spin_timeout_ns; /* budget of each main-loop mbarrier wait of the streamed symmetric
                                apply and the warp-specialised tensor-core block GEMM, in ns,
                                counted as SM clock cycles at the device's maximum clock

@@ -198,7 +198,7 @@ struct feti_ctx {
   // autotuner picked for their apply (0: the FP64 rows are faster)
   int64_t fix_elems[2] = {0, 0};
   int2* d_fix[2] = {nullptr, nullptr};
-  int* d_fixexp[2] = {nullptr, nullptr};
+  int2* d_fixexp[2] = {nullptr, nullptr};
   int fix64[2] = {0, 0};
   bool fix_dropped = false;  // given back for want of memory
   bool ops_ready = false;    // every operator array is allocated
@@ -1970,7 +1970,8 @@ void gemv_apply(feti_ctx* ctx, int which, const int* done, bool f32, const void*
   if (!f32 && ctx->fix64[which]) {
     (void)feti::launch_symv_fixed(ctx->fix64[which], ctx->P, ctx->d_sym_order[which], ctx->sym_max_m[which],
                                   ctx->d_lay, which, ctx->d_fix[which], ctx->d_fixexp[which],
-                                  static_cast<const double*>(v), yo, done, ctx->stream);
+                                  which == 0 ? ctx->d_F : ctx->d_S, static_cast<const double*>(v), yo, done,
+                                  ctx->stream);
     return;
   }
   if (f32 && ctx->sym32[which] == 64 && !ctx->opt.per_subdomain) {
@@ -2187,7 +2188,8 @@ feti_status autotune_run(feti_ctx* ctx) {
         for (int rep = -1; rep < 3; ++rep) {
           if (rep == 0) FETI_CK(cudaEventRecord(e0, st));
           FETI_CK(feti::launch_symv_fixed(C, ctx->P, ctx->d_sym_order[w], ctx->sym_max_m[w], ctx->d_lay, w, ctx->d_fix[w],
-                                          ctx->d_fixexp[w], ctx->d_vloc, ctx->d_loc, ctx->d_zero, st));
+                                          ctx->d_fixexp[w], w == 0 ? ctx->d_F : ctx->d_S, ctx->d_vloc, ctx->d_loc,
+                                          ctx->d_zero, st));
         }
         FETI_CK(cudaEventRecord(e1, st));
         FETI_CK(cudaEventSynchronize(e1));

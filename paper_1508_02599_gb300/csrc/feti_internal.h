@@ -223,16 +223,17 @@ void launch_symv3_f32(int G, int P, const int32_t* order, int max_m, const SubLa
 // lower block triangle in 56-bit fixed point (feti_symv_fixed.cu).
 // launch_fix_operator: row exponents (ex, boundary offsets) and panels out of
 // the full FP64 matrices; launch_symv_fixed: y = M v with C CTAs per
-// subdomain (1, 2, 4 or 8), order: subdomains largest first;
+// subdomain (1, 2, 4 or 8), rows that the fixed point holds too coarsely from the
+// full FP64 matrices M64; order: subdomains largest first;
 // fix_entries: entries of the panels of an operator of m rows;
 // symv_fixed_fits: whether operators up to max_m rows can be applied.
 int64_t fix_entries(int m);
 bool symv_fixed_fits(int max_m);
-void launch_fix_operator(int P, int max_m, const SubLayout* lay, int which, const double* M, int* ex, int2* out,
+void launch_fix_operator(int P, int max_m, const SubLayout* lay, int which, const double* M, int2* ex, int2* out,
                          cudaStream_t st);
 cudaError_t launch_symv_fixed(int C, int P, const int32_t* order, int max_m, const SubLayout* lay, int which,
-                              const int2* M, const int* ex, const double* vloc, double* y, const int* done,
-                              cudaStream_t st);
+                              const int2* M, const int2* ex, const double* M64, const double* vloc, double* y,
+                              const int* done, cudaStream_t st);
 // FP32 signed gather (input of the FP32 apply).
 void launch_gather32(const Maps& mp, const double* x, const double* wv, float* y, const int* done, cudaStream_t st);
 // a += b
