@@ -1314,7 +1314,7 @@ __global__ void __launch_bounds__(SYM_WPC * 32) k_symv2_f32(const int32_t* __res
 
 // y[c] += sum over the panels I below row c (I = c/PH + 1, ..) of their
 // transposed products at column c, in that order.
-__global__ void k_symv_fix(Maps mp, const SubLayout* __restrict__ lay, int which, const float* __restrict__ part,
+__global__ void k_symv_fix(Maps mp, const SubLayout* __restrict__ lay, int which, const float* part,
                            double* __restrict__ y, const int* __restrict__ done) {
   dep_wait();
   dep_go();
@@ -1332,14 +1332,15 @@ __global__ void k_symv_fix(Maps mp, const SubLayout* __restrict__ lay, int which
     const float* ps = part + L.psym;
     // FP32 sum in panel order (the partials carry the FP32 operator's rounding;
     // FP64 adds and conversions would occupy GB300's narrow FP64 pipe), loads
-    // requested sixteen at a time, one FP64 addition to y
+    // requested sixteen at a time, one FP64 addition to y.  The previous kernel
+    // writes the partials: no read-only loads
     float t = 0.f;
     for (int I0 = c / PH + 1; I0 < nP; I0 += 16) {
       float f[16];
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
         const int I = I0 + u;
-        f[u] = I < nP ? __ldg(ps + (size_t)(PH / 2) * I * (I - 1) + c) : 0.f;
+        f[u] = I < nP ? ps[(size_t)(PH / 2) * I * (I - 1) + c] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < 16; ++u) t += f[u];
