@@ -46,7 +46,7 @@ def build(folder):
             f.write(f'long stub{k}(void) __asm__("{name}");\nlong stub{k}(void) {{ return {body}; }}\n')
     lib = os.path.join(folder, "libfeti_fake.so")
     subprocess.run(["gcc", "-fPIC", "-O1", "-c", stub, "-o", stub + ".o"], check=True)
-    subprocess.run(["g++", "-shared", "-Wl,--no-undefined", "-o", lib, *objs, stub + ".o", "-pthread"], check=True)
+    subprocess.run(["g++", "-shared", "-Wl,--no-undefined,-Bsymbolic", "-o", lib, *objs, stub + ".o", "-pthread"], check=True)
     return lib
 
 
