@@ -200,6 +200,7 @@ struct feti_ctx {
   int2* d_fix[2] = {nullptr, nullptr};
   int2* d_fixexp[2] = {nullptr, nullptr};
   int fix64[2] = {0, 0};
+  bool col64[2] = {false, false};  // FP64 block products column by column through it
   bool fix_dropped = false;  // given back for want of memory
   bool ops_ready = false;    // every operator array is allocated
   // symmetric FP32 local applies: lower block-triangles, transposed-product
@@ -2641,8 +2642,6 @@ feti_status write_displacement(feti_ctx* ctx, double* u_out, int on_device, doub
 
 // ---------------------------------------------------------------------------
 // Block form: nrhs right-hand sides share every operator apply.
-// Times the block-form local GEMM schedules (rows per warp step {1, 2, 4},
-// rows per CTA {32, 64}) on the real operators and keeps the fastest.
 // One 2-D tensor map per subdomain over its FP32 copy of F_i (which 0) or of
 // the preconditioner block (which 1): (columns, rows) = (m, m), row pitch the
 // padded stride, 32 x 128 boxes, 128-byte swizzle, out-of-range elements
@@ -2678,6 +2677,12 @@ feti_status build_tensor_maps(feti_ctx* ctx) {
   return FETI_OK;
 }
 
+void apply_columns(feti_ctx* ctx, int which, int nrhs, const int* done);
+
+// Times the block-form local GEMM schedules (rows per warp step {1, 2, 4},
+// rows per CTA {32, 64}) on the real operators, the tensor-core kernels (FP32)
+// and the columns one by one (FP64, where the fixed-point form was picked), and
+// keeps the fastest.
 feti_status autotune_m(feti_ctx* ctx, int nrhs) {
   if (ctx->tuned_m == nrhs) return FETI_OK;
   cudaStream_t st = ctx->stream;
@@ -2713,6 +2718,17 @@ feti_status autotune_m(feti_ctx* ctx, int nrhs) {
             FETI_CK(cudaEventElapsedTime(&ms, e0, e1));
             if (ms < bt) { bt = ms; best = c; }
           }
+        if (!f32 && ctx->fix64[w]) {
+          // once: nrhs products in a row are long enough to time
+          apply_columns(ctx, w, 1, ctx->d_zero);
+          FETI_CK(cudaEventRecord(e0, st));
+          apply_columns(ctx, w, nrhs, ctx->d_zero);
+          FETI_CK(cudaEventRecord(e1, st));
+          FETI_CK(cudaEventSynchronize(e1));
+          float ms = 0.f;
+          FETI_CK(cudaEventElapsedTime(&ms, e0, e1));
+          ctx->col64[w] = 3.0f * ms < bt || ctx->opt.symmetric >= 2;
+        }
         if (f32 && ctx->opt.no_tensor_cores != 1) {
           // tensor-core candidate: kept only if faster and no bounded wait timed out
           if (!ctx->d_tc_err) FETI_TRY(dev_alloc(ctx, &ctx->d_tc_err, 1));
@@ -2780,6 +2796,17 @@ feti_status alloc_multi(feti_ctx* ctx, int nrhs) {
   return autotune_m(ctx, nrhs);
 }
 
+// FP64 block product of dm_vloc into dm_loc, column by column through the
+// single-vector form.
+void apply_columns(feti_ctx* ctx, int which, int nrhs, const int* done) {
+  const int nb = (int)ctx->nb_total;
+  for (int k = 0; k < nrhs; ++k) {
+    feti::launch_col_get(nb, nrhs, k, ctx->dm_vloc, ctx->d_vloc, ctx->stream);
+    gemv_apply(ctx, which, done, false, nullptr, nullptr);
+    feti::launch_col_set(nb, nrhs, k, 1.0, ctx->d_loc, ctx->dm_loc, ctx->stream);
+  }
+}
+
 // Y = W B M B^T W X on blocks (which 0: F_i, no weights; which 1: preconditioner).
 void local_apply_m(feti_ctx* ctx, int which, int nrhs, const double* x, const double* wv, const int* done, bool f32) {
   cudaStream_t st = ctx->stream;
@@ -2798,16 +2825,12 @@ void local_apply_m(feti_ctx* ctx, int which, int nrhs, const double* x, const do
                       : (which == 0 ? (const void*)ctx->d_F : (const void*)ctx->d_S);
   void* v = f32 ? (void*)ctx->dm_vloc32 : (void*)ctx->dm_vloc;
   feti::launch_gather_m(ctx->maps, nrhs, x, wv, v, f32 ? 1 : 0, done, st);
-  if (!f32 && ctx->fix64[which]) {
-    // column by column where the fixed-point form beats the plain apply: the
-    // products of the block kernel occupy the FP64 pipe nrhs times as long (128
-    // subdomains, 8 columns: 1.42 ms against 0.78)
-    const int nb = (int)ctx->nb_total;
-    for (int k = 0; k < nrhs; ++k) {
-      feti::launch_col_get(nb, nrhs, k, ctx->dm_vloc, ctx->d_vloc, st);
-      gemv_apply(ctx, which, done, false, nullptr, nullptr);
-      feti::launch_col_set(nb, nrhs, k, 1.0, ctx->d_loc, ctx->dm_loc, st);
-    }
+  if (!f32 && ctx->fix64[which] && ctx->col64[which]) {
+    // the products of the block kernel occupy the FP64 pipe nrhs times as long
+    // (128 subdomains, 8 columns: 1.42 ms against 0.78), the columns take three
+    // launches each (64 sub-cubes of 125 nodes, 16 columns: solve 29.8 ms against
+    // 26.5): autotune_m times both
+    apply_columns(ctx, which, nrhs, done);
     return;
   }
   if (f32 && ctx->tc_m[which])

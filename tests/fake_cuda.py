@@ -25,7 +25,7 @@ def cuda_include():
 
 
 def build(folder):
-    """The library's path; every undefined launcher returns zero, the fixed-point apply asks the fake."""
+    """The library's path; every undefined launcher returns zero, the local products ask the fake."""
     inc = ["-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", cuda_include(),
            "-I", "/usr/local/cuda/include"]
     jobs, objs = [], []
@@ -40,9 +40,10 @@ def build(folder):
 
     stub = os.path.join(folder, "stubs.c")
     with open(stub, "w") as f:
-        f.write("long fake_fixed_launch(void);\n")
+        fakes = {"launch_symv_fixed": "fixed", "launch_gemv_loc": "rows", "launch_gemm_loc": "block"}
+        f.write("".join(f"long fake_{v}_launch(void);\n" for v in fakes.values()))
         for k, name in enumerate(sorted(names("--undefined-only") - names("--defined-only"))):
-            body = "fake_fixed_launch()" if "launch_symv_fixed" in name else "0"
+            body = next((f"fake_{v}_launch()" for n, v in fakes.items() if n in name), "0")
             f.write(f'long stub{k}(void) __asm__("{name}");\nlong stub{k}(void) {{ return {body}; }}\n')
     lib = os.path.join(folder, "libfeti_fake.so")
     subprocess.run(["gcc", "-fPIC", "-O1", "-c", stub, "-o", stub + ".o"], check=True)
@@ -59,6 +60,7 @@ def load(path):
         _lib._lib = real
     lib.fake_live_bytes.restype = lib.fake_peak_bytes.restype = C.c_size_t
     lib.fake_capacity.argtypes = [C.c_size_t]
+    lib.fake_cost.argtypes = [C.c_float] * 3
     return lib
 
 

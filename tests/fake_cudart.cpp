@@ -17,6 +17,8 @@ std::map<void*, size_t> live;   // device allocations
 size_t live_bytes = 0, peak_bytes = 0, capacity = (size_t)-1;
 int refuse = 0;                 // 1: launches of the fixed-point apply are refused while a stream is captured
 int capturing = 0, graphs = 0, graph_launches = 0, fixed_launches = 0;
+float cost[3] = {};             // of the fixed-point, row and block products' launches
+float now = 0.0f;               // the costs of what was launched
 cudaError_t fail(cudaError_t e) { return last = e; }
 }  // namespace
 
@@ -26,8 +28,10 @@ void fake_reset() {
   capacity = (size_t)-1;
   peak_bytes = live_bytes;
   refuse = capturing = graphs = graph_launches = fixed_launches = 0;
+  cost[0] = cost[1] = cost[2] = 0.0f;
 }
 void fake_capacity(size_t bytes) { capacity = bytes; }
+void fake_cost(float fixed, float rows, float block) { cost[0] = fixed, cost[1] = rows, cost[2] = block; }
 void fake_refuse_in_capture(int on) { refuse = on; }
 size_t fake_live_bytes() { return live_bytes; }
 size_t fake_peak_bytes() { return peak_bytes; }
@@ -36,8 +40,11 @@ int fake_count(int what) { return what == 0 ? graphs : what == 1 ? graph_launche
 
 feti_status feti_dual_apply_noalloc(feti_ctx*, const double*, double*, double*) { return FETI_ERR_STATE; }
 
+long fake_rows_launch() { return now += cost[1], 0; }
+long fake_block_launch() { return now += cost[2], 0; }
 long fake_fixed_launch() {
   ++fixed_launches;
+  now += cost[0];
   return refuse && capturing ? fail(cudaErrorInvalidValue) : cudaSuccess;
 }
 
@@ -96,13 +103,13 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long 
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { std::free(g); return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { std::free(e); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { ++graph_launches; return capturing ? fail(cudaErrorIllegalState) : cudaSuccess; }
-cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)std::malloc(1); return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)std::calloc(1, sizeof(float)); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { std::free(e); return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { *(float*)e = now; return cudaSuccess; }
 cudaError_t cudaEventRecordWithFlags(cudaEvent_t, cudaStream_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) { *ms = 1.0f + *(float*)b - *(float*)a; return cudaSuccess; }
 cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult*) {
   *f = nullptr;
   return fail(cudaErrorInvalidValue);

@@ -105,3 +105,18 @@ def test_set_up_that_ran_out_of_memory_is_completed_by_the_next(lib, monkeypatch
         lib.fake_capacity(2 ** 62)
         s.prepare()
         assert lib.fake_live_bytes() == full
+
+
+@pytest.mark.parametrize("symmetric,block,columns", [("auto", 3.0, False), ("auto", 6.0, True), ("force", 3.0, True)])
+def test_block_products_take_the_faster_form(lib, monkeypatch, symmetric, block, columns):
+    """Two columns of cost 2 through the fixed-point copy, or one block launch."""
+    prob = mesh.cube_problem(4, (2, 2, 1))                      # the picks of _prob() are known by now
+    with fake_cuda.solver(lib, monkeypatch, prob, method="af", symmetric=symmetric, maxit=20) as s:
+        lib.fake_cost(2.0, 9.0, block)
+        s.prepare()
+        assert s.schedule()["fp64_M"][0] <= -400               # the tuner's pick for one vector
+        v, q, z = (np.zeros((s.sizes()["n_lambda"], 2)) for _ in range(3))
+        fake_cuda.dual_apply(lib, s, v, q, z, 2)               # tunes the block form
+        launched = lib.fake_count(FIXED)
+        fake_cuda.dual_apply(lib, s, v, z, q, 2)               # captured anew: F v as a block, then the preconditioner
+        assert lib.fake_count(FIXED) - launched == (2 if columns else 0)
