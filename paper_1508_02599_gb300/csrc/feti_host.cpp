@@ -3833,11 +3833,10 @@ feti_status feti_dual_apply(feti_ctx* ctx, const double* v, double* q, double* z
   }
   ctx->gemv_ms = kern / n_apply;
   // algorithmic bytes of one F_i apply: the n(n+1)/2 distinct entries of the
-  // symmetric F_i once (8 B in FP64, 7 B in its fixed-point form, 4 B in the
-  // FP32 copy), the gathered
-  // local input (8 B) and the local output (8 B) per boundary DOF; flops: 2
-  // per entry of the full matrix
-  const double esz = f32_ops(ctx) ? 4.0 : ctx->fix64[0] ? 7.0 : 8.0;
+  // symmetric F_i once (8 B in FP64 and in its fixed-point form, 4 B in the
+  // FP32 copy), the gathered local input (8 B) and the local output (8 B) per
+  // boundary DOF; flops: 2 per entry of the full matrix
+  const double esz = f32_ops(ctx) ? 4.0 : 8.0;
   ctx->gemv_bytes = half * esz + vec * 16.0;
   ctx->gemv_flops = 2.0 * entries;
   return FETI_OK;

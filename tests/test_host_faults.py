@@ -120,3 +120,15 @@ def test_block_products_take_the_faster_form(lib, monkeypatch, symmetric, block,
         launched = lib.fake_count(FIXED)
         fake_cuda.dual_apply(lib, s, v, z, q, 2)               # captured anew: F v as a block, then the preconditioner
         assert lib.fake_count(FIXED) - launched == (2 if columns else 0)
+
+
+def test_bytes_of_an_apply_are_those_stored(lib, monkeypatch):
+    """An entry takes 8 bytes in the FP64 rows and in the fixed-point copy."""
+    moved = []
+    for symmetric in ("off", "force"):
+        with fake_cuda.solver(lib, monkeypatch, _prob(), method="af", symmetric=symmetric, maxit=20) as s:
+            s.prepare()
+            n = s.sizes()["n_lambda"]
+            fake_cuda.dual_apply(lib, s, *(np.zeros(n) for _ in range(3)))
+            moved.append(s.kernel_stats()["gemv_bytes"])
+    assert moved[0] == moved[1] > 0
