@@ -555,8 +555,10 @@ def main():
                 blk[name] = {k: v for k, v in b.items() if k not in ("U", "scales")}
                 blk[name]["max_rel_err_vs_single_fp64"] = max(errs)
             blk["fp32_local"]["gemm_hbm_frac"] = blk["fp32_local"]["gemm_gbs"] / peaks["hbm_gbs"]
-            blk["note"] = ("16 load cases (pressure x U[8,16], seeded) solved as one block: every dense F_i/S_i "
-                           "entry read feeds 16 products; rhs_applies_per_s counts right-hand sides")
+            blk["note"] = ("16 load cases (pressure x U[8,16], seeded) solved as one block; rhs_applies_per_s counts "
+                           "right-hand sides.  An entry of F_i/S_i that is read feeds 16 products in the FP32 form and "
+                           "in the FP64 F_i product of rhs_applies_per_s; the other FP64 products go column by column "
+                           "through the fixed-point copy where that is faster")
             line["block16"] = blk
         if args.elements:
             line["elements"] = measure_elements()

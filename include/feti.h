@@ -378,6 +378,10 @@ feti_status feti_dual_apply_multi(feti_ctx* ctx, const double* v, double* q, dou
  *    without waiting.  All calls share the array: calls whose work overlaps
  *    on the GPU (other streams, other contexts) race on it.  Every scratch
  *    entry is written before it is read, so nothing needs clearing.
+ *  - FP64 operators are applied by rows here, as with feti_options.symmetric = 1:
+ *    where feti_dual_apply takes the fixed-point copy the two differ in their
+ *    last bits, and this call is the slower one (it is for what it does not
+ *    allocate, not for speed).
  *  - Requires feti_prepare (or feti_solve) on this context first. */
 feti_status feti_dual_apply_noalloc(feti_ctx* ctx, const double* v, double* q, double* z);
 

@@ -4,7 +4,7 @@
 //
 // Design for GB300: FP64 arithmetic issues at about two FMAs per clock per SM,
 // so every FP64 kernel here is bounded by the FP64 pipe or by HBM; gathers are
-// row-major and deterministic (no floating-point atomics anywhere); every
+// row-major and deterministic (no floating-point atomics here); every
 // subdomain of uneven size is one batch element of a single launch.
 #include "feti_internal.h"
 #include "feti_launch.cuh"
@@ -2551,8 +2551,8 @@ __global__ void k_lump_fill(long nnz, const int64_t* __restrict__ src, const T* 
     val[j] = A[src[j]];
 }
 
-// y = K_bb v on every subdomain's boundary positions, one warp per row.
-// Four lanes per row: of a warp per row's seven FP64 instructions five were the
+// y = K_bb v on every subdomain's boundary positions, four lanes per row: of a
+// warp per row's seven FP64 instructions five were the
 // sum over the lanes.  A batch of 16 entries of each row is loaded at once, the
 // first before the wait (the pattern and the values are the setup's).  128
 // subdomains: 29.4 -> 11.4 us.

@@ -24,9 +24,9 @@ namespace {
 // visible.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel's CTAs be placed (once every CTA of this one has said so
-// or ended).  The large local applies neither say it nor are launched this way:
-// waiting CTAs beside them, or CTAs of theirs placed unevenly beside the
-// gather, cost more than the launch.
+// or ended).  Large operators' fixed-point applies (launch_symv_fixed) neither
+// say it nor are launched this way: waiting CTAs beside them, or CTAs of theirs
+// placed unevenly beside the gather, cost more than the launch.
 __device__ __forceinline__ void dep_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename T>
 __device__ __forceinline__ T* fresh(T* p) {

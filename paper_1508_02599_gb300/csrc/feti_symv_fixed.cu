@@ -459,11 +459,12 @@ cudaError_t launch_fix(int C, int P, const int32_t* order, int max_m, const SubL
 
 }  // namespace
 
-// Shared memory of the largest operator, and row sums of at most 64 tiles
-// (2^63 / 2^56 / 2 columns a lane) in 64 bits.
 int64_t fix_entries(int m) { return fix_panel((m + PR - 1) / PR); }
 
-bool symv_fixed_fits(int max_m) { return fix_smem(max_m, 8) <= kFixSmem && max_m <= 4032; }
+// Shared memory of the largest operator: up to 3,200 rows.  The row sums would
+// hold in 64 bits up to 64 tiles (2^63 / 2^56 / 2 columns a lane).
+static_assert(kFixSmem / (sizeof(int2) + 8 * sizeof(double)) < 64 * 64 - PR, "row sums of one row's tiles in 64 bits");
+bool symv_fixed_fits(int max_m) { return fix_smem(max_m, 8) <= kFixSmem; }
 
 void launch_fix_operator(int P, int max_m, const SubLayout* lay, int which, const double* M, int2* ex, int2* out,
                          cudaStream_t st) {
@@ -477,7 +478,7 @@ cudaError_t launch_symv_fixed(int C, int P, const int32_t* order, int max_m, con
                               const int* done, cudaStream_t st) {
   // six warps and two CTAs per SM, so that one CTA's start and end run beside
   // the other's stream, while two sets of buffers fit
-  if (2 * fix_smem(max_m, 6) <= kFixSmem) 
+  if (2 * fix_smem(max_m, 6) <= kFixSmem)
     return launch_fix<6>(C, P, order, max_m, lay, which, M, ex, M64, vloc, y, done, st);
   return launch_fix<8>(C, P, order, max_m, lay, which, M, ex, M64, vloc, y, done, st);
 }
